@@ -181,13 +181,15 @@ typedef struct sesw_info {
     int32_t patch_vertices;  /* target vertices per patch */
     int32_t block_threads;   /* threads per block of the substep (or persistent) kernel */
     int32_t mode;            /* SESW_MODE_GRAPH or SESW_MODE_PERSISTENT (0 from sesw_mesh_check) */
-    int32_t blocks_per_sm;   /* persistent mode: resident blocks per SM */
+    int32_t blocks_per_sm;   /* persistent mode: resident blocks per SM (the register SE kernel: teams of
+                                block_threads threads, each with its patch, in one block per SM) */
     int32_t slots_per_thread;/* persistent mode: element slots per thread (held in registers,
                                 or slot-loop rounds when streamed) */
-    int32_t cached;          /* persistent mode, register kernels: 1 when the static slot data lives in
-                                shared memory, 2 when the vertices' data and the low parts of the
-                                compensated sums do and the static slot data are read from L2
-                                (large patches); streaming kernels (streamed != 0): 1 when the
+    int32_t cached;          /* persistent mode, register kernels: 1 when the patch's static data lives on
+                                chip (vertices' data in shared memory, slots' in tensor memory; the
+                                SESM kernel: all in shared memory), 2 when all but some of the slots'
+                                forcing and corner indices does, the low parts of the compensated sums
+                                in shared memory (large patches); 0: read from L2; streaming kernels (streamed != 0): 1 when the
                                 vertices' data lives in shared memory */
     int32_t nbasin;          /* meshes in the uploaded batch (1 for sesw_mesh_upload) */
     double courant_max;      /* estimated largest substep Courant number sqrt(gH kappa^2) dt
@@ -269,8 +271,8 @@ int sesw_set_mode(sesw_ctx *ctx, int32_t mode);
 int sesw_set_persistent_form(sesw_ctx *ctx, int32_t form);
 
 /* Persistent mode, batches: the residency and kernel form of the packs of "large" basins,
- * those too large for one grid of patches of the common size (the largest patch whose static
- * data fits shared memory at the batch's blocks per SM, 1280 vertices at one block per SM).
+ * those too large for one grid of patches of the common size (1280 vertices at one block per SM,
+ * 1280 / k at k).
  * Such a basin fills its own grid of blocks_per_sm x SMs patches; blocks_per_sm 0 (default)
  * takes the batch's own value, and form -1 (default) the form of sesw_set_persistent_form.
  * With two blocks per SM and the streaming form, for example, a 400k-vertex basin runs 304

@@ -603,6 +603,7 @@ int build_halos(HostMesh &hm, std::string &err)
     hm.patch_halo.assign(np + 1, 0);
     hm.halo_v.clear();
     hm.slot_l.assign(hm.nslot, make_ushort4(0, 0, 0, 0));
+    hm.slot_f.assign(hm.nslot, make_uint2(0xffffffffu, 0x7fffffffu));
     hm.max_patch_local = 0;
     hm.max_patch_halo = 0;
     hm.max_patch_csr = 0;
@@ -635,6 +636,18 @@ int build_halos(HostMesh &hm, std::string &err)
             }
             hm.slot_l[s] = make_ushort4(l[0], l[1], l[2], 0);
         }
+        // where each corner's flux goes: the own vertex it belongs to and its place in that
+        // vertex's incidence order, 21 bits per corner (HostMesh::slot_f)
+        for (int v = vlo; v < vhi; v++)
+            for (int k = hm.vcsr_off[v]; k < hm.vcsr_off[v + 1] && k - hm.vcsr_off[v] < 16; k++) {
+                const uint32_t q = hm.vcsr[k];
+                uint2 &f = hm.slot_f[hm.patch_slot[p] + (int)(q >> 2)];
+                const int c = (int)(q & 3u);
+                uint64_t w = ((uint64_t)f.y << 32) | f.x;
+                const uint64_t e = ((uint64_t)(v - vlo) << 4) | (uint64_t)(k - hm.vcsr_off[v]);
+                w = (w & ~(0x1fffffull << (21 * c))) | (e << (21 * c));
+                f = make_uint2((uint32_t)w, (uint32_t)(w >> 32));
+            }
         hm.halo_v.insert(hm.halo_v.end(), halo.begin(), halo.end());
         hm.patch_halo[p + 1] = (int)hm.halo_v.size();
         hm.max_patch_local = std::max(hm.max_patch_local, nloc);

@@ -120,12 +120,14 @@ int capture_step_graph(sesw_ctx *c, int parity, cudaGraphExec_t *out)
     cudaGraph_t g = nullptr;
     CK(c, cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t e = cudaSuccess;
-    if (c->ds.eta_sum) e = cudaMemsetAsync(c->ds.eta_sum, 0, sizeof(float) * (size_t)c->dm.nv, c->cap_stream);
+    // (the persistent kernels start the sum themselves)
+    if (c->ds.eta_sum && c->mode != SESW_MODE_PERSISTENT)
+        e = cudaMemsetAsync(c->ds.eta_sum, 0, sizeof(float) * (size_t)c->dm.nv, c->cap_stream);
     if (e != cudaSuccess) {
     } else if (c->mode == SESW_MODE_PERSISTENT) {
         e = c->params.scheme == 1
                 ? sesw::launch_persistent_sesm(c->dm, c->ds, c->args, c->params.M, parity, c->packs, c->cap_stream)
-                : sesw::launch_persistent(c->dm, c->ds, c->args, c->params.M, parity, c->groups, c->cap_stream);
+                : sesw::launch_persistent(c->dm, c->ds, c->args, c->params.M, parity, 1, c->groups, c->cap_stream);
     } else if (c->params.scheme == 1) {
         // SESM: level rings, U^m in B[m % 3] (B[0] holds U^0 and, at the end, U^M) and
         // eta^m in Er[m % 5] (Er[0] holds eta^0 and, at the end, eta^M); levels before
@@ -203,7 +205,7 @@ int enqueue_step(sesw_ctx *c)
         if (c->params.scheme == 1)
             CK(c, sesw::launch_persistent_sesm(c->dm, c->ds, c->args, c->params.M, c->parity, c->packs, c->stream));
         else
-            CK(c, sesw::launch_persistent(c->dm, c->ds, c->args, c->params.M, c->parity, c->groups, c->stream));
+            CK(c, sesw::launch_persistent(c->dm, c->ds, c->args, c->params.M, c->parity, 1, c->groups, c->stream));
         c->parity ^= 1;
         return SESW_OK;
     }
@@ -414,7 +416,7 @@ static int prepare_parts(sesw_ctx *c, const sesw_mesh *meshes, int n, const std:
 // patches). In a batch every basin must fit one grid, and basins are packed whole into
 // packs of at most nblk patches, one cooperative launch each: a basin gets the larger of
 // its one-grid size and a common size `base`, the largest patch whose static data fits
-// shared memory (so most basins run the cached kernel), or a smaller one when the whole
+// on chip in every scheme's kernel, or a smaller one when the whole
 // batch then fits a single pack. Basins whose one-grid size exceeds `base` ("large") are
 // cut into one grid of nblk_large patches instead (their own residency, see
 // sesw_set_large_basins) and marked in `large`. Returns base.
@@ -761,6 +763,7 @@ static int upload_batch(sesw_ctx *c, const sesw_mesh *meshes, int n)
         TRY(upload(c, &d.patch_halo, hm.patch_halo, "patch_halo"));
         TRY(upload(c, &d.halo_v, hm.halo_v, "halo_v"));
         TRY(upload(c, &d.slot_l, hm.slot_l, "slot_l"));
+        TRY(upload(c, &d.slot_f, hm.slot_f, "slot_f"));
         d.max_patch_local = hm.max_patch_local;
         d.max_patch_vertices = hm.max_patch_vertices;
         d.max_patch_halo = hm.max_patch_halo;

@@ -72,6 +72,8 @@ struct HostMesh {
     std::vector<int> patch_halo;   // [npatch+1] ranges into halo_v
     std::vector<int> halo_v;       // halo vertex ids (new order), sorted per patch
     std::vector<ushort4> slot_l;   // local corner indices of each slot (.w unused)
+    std::vector<uint2> slot_f;     // per corner 21 bits (corner 0 lowest): own local vertex << 4 | the corner's
+                                   // place in that vertex's incidences; all ones: not an own vertex (or place > 15)
     int max_patch_local = 0;       // max n_own + n_halo
     int max_patch_halo = 0;        // max n_halo
     int max_patch_csr = 0;         // max incidence entries of one patch's own vertices
@@ -141,6 +143,7 @@ struct DevMesh {
     int *patch_halo = nullptr;
     int *halo_v = nullptr;
     ushort4 *slot_l = nullptr;
+    uint2 *slot_f = nullptr;
     int max_patch_local = 0, max_patch_vertices = 0, max_patch_halo = 0, max_patch_csr = 0;
 };
 
@@ -241,7 +244,12 @@ cudaError_t launch_diagnostics_basins(const DevMesh &m, const DevState &s, const
 struct PersistentPlan {
     int slots_per_thread = 0;   // 0: not possible for this mesh
     int threads = 0;
-    int cached = 0;             // 1: the patch's static data lives in shared memory
+    int cached = 0;             // 1: the patch's static data lives on chip (vertices' data in shared memory,
+                                // slots' in tensor memory; the SESM kernel: all in shared memory); 2: the same
+                                // except some of the slots' forcing and corner indices, read from L2
+    // the register SE kernel: a block per SM of `teams` teams, each with `threads` threads and its
+    // part of the shared memory; at most `grid` blocks, with tmem_cols tensor-memory columns each
+    int teams = 1, team_smem = 0, tmem_cols = 0, grid = 0;
     int stream = 0;             // state and static data in global memory (the streaming kernels):
                                 // 1 with the corner indices in shared memory, 2 without
     int blocks_per_sm = 1;
@@ -270,8 +278,9 @@ struct PackGroup {
 PersistentPlan persistent_plan(const PatchMax &mx, int blocks_per_sm);
 cudaError_t persistent_prepare(const PersistentPlan &plan);
 size_t persistent_flag_bytes(int npatch);
+// One launch per group advances its packs nsteps steps (1 where a group streams its state).
 cudaError_t launch_persistent(const DevMesh &m, const DevState &s, const StepArgs &a, int M, int parity,
-                              const std::vector<PackGroup> &groups, cudaStream_t stream);
+                              int nsteps, const std::vector<PackGroup> &groups, cudaStream_t stream);
 // The SESM scheme for patches too large for its on-chip state (k_persistent_sesm_stream):
 // two more slot arrays (DevState::U_x) hold U^{m-2} and U_AB^{m-1}.
 // idx_mode: -1 keeps the slots' corner indices in shared memory when they fit, 0 never.

@@ -46,6 +46,7 @@ struct PArgs {
     const uint32_t *vcsr;
     const int4 *sv;
     const ushort4 *sl;
+    const uint2 *sf;           // where each corner's flux goes (DevMesh::slot_f)
     const float4 *sg, *sc;
     const float4 *sk;          // step coefficients of each slot (DevMesh::slot_k)
     const float2 *R;
@@ -65,6 +66,11 @@ struct PArgs {
     int pack_first, pack_last;   // launches of a group of packs (the SE kernels)
     StepArgs a;
     int M, npatch;
+    int nsteps;                  // baroclinic steps of this launch (k_persistent)
+    unsigned tmem_cols;          // tensor-memory columns of a block (k_persistent, a power of two)
+    int row_quads, row_vertices; // k_persistent: 16-byte quads of a vertex's row of fluxes; vertices per quad array
+    int off_dummy, off_f01, off_f2, off_slo;   // k_persistent: see SeLayout
+    int team_threads, team_smem; // threads and shared-memory bytes of each patch of a block (k_persistent)
     // shared-memory carve-up (CACHED), in bytes from the dynamic shared base
     int off_flux, off_g, off_c, off_r, off_l, off_off, off_csr, off_inv, off_halo;
     // inc8: the cached incidences are one row of 8 16-bit byte offsets per own vertex (into the
@@ -120,17 +126,255 @@ __device__ __forceinline__ float halo_eta(const PArgs &P, const unsigned long lo
     return 0.0f;
 }
 
+// ---------------------------------------------------------------------------------
+// Tensor memory as the store of the slots' static data. An SM has 256 KB of it beside the
+// 256 KB of registers and 228 KB of shared memory: 64 words for each of 1024 threads. A warp
+// reads and writes only its own 32 lanes (32 (w % 4) .. + 31), which suits data that
+// belongs to one thread: word k of a thread is its lane of column base + k. A tcgen05.ld of
+// 8 words costs the shared-memory pipe nothing, where the same words from shared memory take
+// 8 of its cycles per warp (the element pass and the vertex pass keep that pipe busy with
+// the gathers of the elevation and the fluxes).
+__device__ __forceinline__ void tmem_alloc(uint32_t *smem_slot, unsigned cols)
+{
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     (uint32_t)__cvta_generic_to_shared(smem_slot)),
+                 "r"(cols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+}
+
+__device__ __forceinline__ void tmem_dealloc(uint32_t base, unsigned cols)
+{
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(base), "r"(cols));
+}
+
+__device__ __forceinline__ void tmem_fence_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tmem_fence_before_sync() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+// Shared memory by 32-bit address (so that no access goes through a generic one); ordered
+// among themselves and by the teams' barriers.
+__device__ __forceinline__ float lds(uint32_t a)
+{
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ float2 lds2(uint32_t a)
+{
+    float2 v;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ float4 lds4(uint32_t a)
+{
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ uint32_t lds_u32(uint32_t a)
+{
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ uint32_t lds_u16(uint32_t a)
+{
+    unsigned short v;
+    asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ void sts(uint32_t a, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v)); }
+__device__ __forceinline__ void sts2(uint32_t a, float2 v)
+{
+    asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y));
+}
+
+__device__ __forceinline__ void tmem_st2(uint32_t t, uint32_t a, uint32_t b)
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1, %2};" ::"r"(t), "r"(a), "r"(b) : "memory");
+}
+
+__device__ __forceinline__ void tmem_st4(uint32_t t, float a, float b, float c, float d)
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(t), "f"(a), "f"(b), "f"(c),
+                 "f"(d)
+                 : "memory");
+}
+
+// A slot's static data: gradients, step coefficients (DevMesh::slot_k), forcing, and the
+// shared-memory addresses of its corners' elevations and of the places of its three fluxes.
+struct SlotData {
+    float4 g, c;
+    float2 r;
+    uint32_t a0, a1, a2, f0, f1, f2;
+};
+
+// The data of one slot as a thread's words hold it, waited for. No memory clobber: what a launch
+// stores in tensor memory is stored before its first barrier and never changes.
+__device__ __forceinline__ void tmem_ld16(uint32_t t, SlotData &q)
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
+                 "%14, %15}, [%16];\n"
+                 "tcgen05.wait::ld.sync.aligned;"
+                 : "=f"(q.g.x), "=f"(q.g.y), "=f"(q.g.z), "=f"(q.g.w), "=f"(q.c.x), "=f"(q.c.y), "=f"(q.c.z),
+                   "=f"(q.c.w), "=f"(q.r.x), "=f"(q.r.y), "=r"(q.a0), "=r"(q.a1), "=r"(q.a2), "=r"(q.f0), "=r"(q.f1),
+                   "=r"(q.f2)
+                 : "r"(t));
+}
+
+__device__ __forceinline__ void tmem_ld12(uint32_t t8, uint32_t t4, SlotData &q, uint32_t &l01, uint32_t &l2)
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%12];\n"
+                 "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%8, %9, %10, %11}, [%13];\n"
+                 "tcgen05.wait::ld.sync.aligned;"
+                 : "=f"(q.g.x), "=f"(q.g.y), "=f"(q.g.z), "=f"(q.g.w), "=f"(q.c.x), "=f"(q.c.y), "=f"(q.c.z),
+                   "=f"(q.c.w), "=f"(q.r.x), "=f"(q.r.y), "=r"(l01), "=r"(l2)
+                 : "r"(t8), "r"(t4));
+}
+
+__device__ __forceinline__ void tmem_ld10(uint32_t t8, uint32_t t2, SlotData &q, uint32_t &l01, uint32_t &l2)
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%10];\n"
+                 "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%8, %9}, [%11];\n"
+                 "tcgen05.wait::ld.sync.aligned;"
+                 : "=f"(q.g.x), "=f"(q.g.y), "=f"(q.g.z), "=f"(q.g.w), "=f"(q.c.x), "=f"(q.c.y), "=f"(q.c.z),
+                   "=f"(q.c.w), "=r"(l01), "=r"(l2)
+                 : "r"(t8), "r"(t2));
+}
+
+__device__ __forceinline__ void tmem_ld8(uint32_t t8, SlotData &q)
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
+                 "tcgen05.wait::ld.sync.aligned;"
+                 : "=f"(q.g.x), "=f"(q.g.y), "=f"(q.g.z), "=f"(q.g.w), "=f"(q.c.x), "=f"(q.c.y), "=f"(q.c.z),
+                   "=f"(q.c.w)
+                 : "r"(t8));
+}
+
+// Where the data of a thread's SPT slots live. Up to 4 slots per thread each slot has 16 words
+// of tensor memory: everything, with the shared-memory offsets ready to use, so that a slot's
+// update spends no instruction on addresses. With 5, 12 words (offsets of the corners packed as
+// 16-bit word indices); with 6, 10 words (without the forcing); with 7 and 8, 8 words and the
+// corners of the first four slots of 7. From 5 slots per thread the places of the fluxes are
+// 16-bit word indices in shared memory; the forcing and corners left over come from L2
+// (coalesced, their addresses known ahead). load is called by whole warps; s is the slot's
+// index in the mesh, i in the patch, team the address of the team's shared memory.
+template <int SPT>
+struct TmemSlots {
+    static constexpr int kWords = SPT <= 4 ? 16 * SPT : (SPT <= 6 ? 60 : 64);
+    static constexpr bool kTmem = true;
+    static constexpr bool kFluxShared = SPT >= 5;
+    __device__ static __forceinline__ void store(uint32_t tm, int j, const SlotData &q)
+    {
+        auto f = [](uint32_t x) { return __uint_as_float(x); };
+        const int b = (SPT <= 4 ? 16 : 8) * j;
+        tmem_st4(tm + b, q.g.x, q.g.y, q.g.z, q.g.w);
+        tmem_st4(tm + b + 4, q.c.x, q.c.y, q.c.z, q.c.w);
+        const uint32_t l01 = (q.a0 >> 2) | (q.a1 << 14), l2 = q.a2;
+        if (SPT <= 4) {
+            tmem_st4(tm + b + 8, q.r.x, q.r.y, f(q.a0), f(q.a1));
+            tmem_st4(tm + b + 12, f(q.a2), f(q.f0), f(q.f1), f(q.f2));
+        } else if (SPT == 5) {
+            tmem_st4(tm + 8 * SPT + 4 * j, q.r.x, q.r.y, f(l01), f(l2));
+        } else if (SPT == 6 || (SPT == 7 && j < 4)) {
+            tmem_st2(tm + 8 * SPT + 2 * j, l01, l2);
+        }
+    }
+    __device__ static __forceinline__ SlotData load(uint32_t tm, int j, const PArgs &P, int s, int i, uint32_t team)
+    {
+        SlotData q;
+        if (SPT <= 4) {
+            tmem_ld16(tm + 16 * j, q);
+            return q;
+        }
+        uint32_t l01, l2;
+        if (SPT >= 6) q.r = __ldg(P.R + s);
+        if (SPT == 5) {
+            tmem_ld12(tm + 8 * j, tm + 8 * SPT + 4 * j, q, l01, l2);
+        } else if (SPT == 6 || (SPT == 7 && j < 4)) {
+            tmem_ld10(tm + 8 * j, tm + 8 * SPT + 2 * j, q, l01, l2);
+        }
+        if (SPT <= 6 || (SPT == 7 && j < 4)) {
+            q.a0 = (l01 & 0xffffu) * 4u;
+            q.a1 = (l01 >> 16) * 4u;
+            q.a2 = l2;
+        } else {
+            const uint2 l = __ldg(reinterpret_cast<const uint2 *>(P.sl + s));
+            tmem_ld8(tm + 8 * j, q);
+            q.a0 = team + (l.x & 0xffffu) * 4u;
+            q.a1 = team + (l.x >> 16) * 4u;
+            q.a2 = team + (l.y & 0xffffu) * 4u;
+        }
+        const uint32_t f01 = lds_u32(team + P.off_f01 + 4 * i);
+        q.f0 = (f01 & 0xffffu) * 4u;
+        q.f1 = (f01 >> 16) * 4u;
+        q.f2 = lds_u16(team + P.off_f2 + 2 * i) * 4u;
+        return q;
+    }
+};
+
+// The same interface with everything read from L2 and the fluxes slot by slot (three words each)
+// at P.off_flux.
+template <int SPT>
+struct GlobalSlots {
+    static constexpr int kWords = 0;
+    static constexpr bool kTmem = false;
+    static constexpr bool kFluxShared = false;
+    __device__ static __forceinline__ void store(uint32_t, int, const SlotData &) {}
+    __device__ static __forceinline__ SlotData load(uint32_t, int, const PArgs &P, int s, int i, uint32_t team)
+    {
+        SlotData q;
+        const ushort4 l = P.sl[s];
+        q.g = P.sg[s];
+        q.c = P.sk[s];
+        q.r = P.R[s];
+        q.a0 = team + 4u * l.x;
+        q.a1 = team + 4u * l.y;
+        q.a2 = team + 4u * l.z;
+        q.f0 = team + (uint32_t)P.off_flux + 12u * (uint32_t)i;
+        q.f1 = q.f0 + 4u;
+        q.f2 = q.f0 + 8u;
+        return q;
+    }
+};
+
+// Tensor-memory columns of a block of `threads` threads with `words` words each: ceil(warps / 4)
+// column groups, rounded up to the allocation unit (a power of two of at least 32).
+inline unsigned tmem_columns(int threads, int words)
+{
+    const int need = ((threads / 32 + 3) / 4) * words;
+    unsigned c = 32;
+    while ((int)c < need) c *= 2;
+    return c;
+}
+
+// Shared memory a block must take so that its share of the SM's shared memory is its share of
+// the SM's 512 tensor-memory columns, less the 1 KB that the system reserves per block and at
+// most 1/32 (and 1 KB) of rounding. Blocks of different launches (other contexts, other streams)
+// may share an SM; columns come in units of 32 = 1/16 of the SM, so blocks that fit its shared
+// memory together always find their columns free, and no resident block can wait for columns
+// that another launch holds.
+inline size_t tmem_smem_floor(unsigned cols, size_t smem_per_sm)
+{
+    const size_t share = smem_per_sm / 512 * cols;
+    return share - 1024 - std::min<size_t>(1024, share / 32);
+}
 
 // Copy the incidences of a patch's own vertices into shared memory (cached layouts): with
 // P.inc8, one row of kIncWidth 16-bit byte offsets (inc8 = 1) or word indices (inc8 = 2) per
 // vertex, pointing at its corner fluxes in incidence order and padded with the zero word; else
-// the CSR with flux indices 3 * slot + corner. Also clears the zero word. The caller synchronises the block afterwards.
-__device__ __forceinline__ void cache_incidences(const PArgs &P, unsigned char *smem_raw, int v0, int nown)
+// the CSR with flux indices 3 * slot + corner. Also clears the zero word. Run by T threads (tid
+// 0 .. T - 1) on the shared memory of one patch; the caller synchronises them afterwards.
+__device__ __forceinline__ void cache_incidences(const PArgs &P, unsigned char *smem_raw, int v0, int nown, int tid,
+                                                 int T)
 {
     const int c0 = P.vcsr_off[v0], ncsr = P.vcsr_off[v0 + nown] - c0;
     if (P.inc8) {
         uint4 *rows = reinterpret_cast<uint4 *>(smem_raw + P.off_off);
-        for (int i = threadIdx.x; i < nown; i += blockDim.x) {
+        for (int i = tid; i < nown; i += T) {
             const int k0 = P.vcsr_off[v0 + i], deg = P.vcsr_off[v0 + i + 1] - k0;
             unsigned h[kIncWidth];
 #pragma unroll
@@ -144,12 +388,12 @@ __device__ __forceinline__ void cache_incidences(const PArgs &P, unsigned char *
             }
             rows[i] = make_uint4(h[0] | (h[1] << 16), h[2] | (h[3] << 16), h[4] | (h[5] << 16), h[6] | (h[7] << 16));
         }
-        if (threadIdx.x == 0) *reinterpret_cast<float *>(smem_raw + P.zero_off) = 0.0f;
+        if (tid == 0) *reinterpret_cast<float *>(smem_raw + P.zero_off) = 0.0f;
     } else {
         unsigned short *s_off = reinterpret_cast<unsigned short *>(smem_raw + P.off_off);
         unsigned short *s_csr = reinterpret_cast<unsigned short *>(smem_raw + P.off_csr);
-        for (int i = threadIdx.x; i <= nown; i += blockDim.x) s_off[i] = (unsigned short)(P.vcsr_off[v0 + i] - c0);
-        for (int k = threadIdx.x; k < ncsr; k += blockDim.x) {
+        for (int i = tid; i <= nown; i += T) s_off[i] = (unsigned short)(P.vcsr_off[v0 + i] - c0);
+        for (int k = tid; k < ncsr; k += T) {
             const uint32_t q = P.vcsr[c0 + k];
             s_csr[k] = (unsigned short)(3u * (q >> 2) + (q & 3u));
         }
@@ -257,6 +501,7 @@ inline PArgs make_pargs(const DevMesh &m, const DevState &s, const StepArgs &a, 
     P.vcsr = m.vcsr;
     P.sv = m.slot_v;
     P.sl = m.slot_l;
+    P.sf = m.slot_f;
     P.sg = m.slot_g;
     P.sc = m.slot_c;
     P.sk = m.slot_k;
@@ -275,6 +520,9 @@ inline PArgs make_pargs(const DevMesh &m, const DevState &s, const StepArgs &a, 
     P.status = s.status;
     P.a = a;
     P.M = M;
+    P.nsteps = 1;
+    P.tmem_cols = 0;
+    P.team_threads = P.team_smem = 0;
     P.npatch = m.npatch;
     const SmemLayout L = smem_layout(mx);
     P.off_flux = L.off_flux;

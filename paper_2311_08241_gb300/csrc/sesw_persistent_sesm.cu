@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(kSesmThreads, 2) k_persistent_sesm(PArgs P)
         s_r[i] = P.R[s0 + i];
         s_l[i] = P.sl[s0 + i];
     }
-    cache_incidences(P, smem_raw, v0, nown);
+    cache_incidences(P, smem_raw, v0, nown, threadIdx.x, T);
     for (int i = threadIdx.x; i < nown; i += T) s_inv[i] = P.inv_av[v0 + i];
     for (int i = threadIdx.x; i < nhalo; i += T) s_halo[i] = P.halo_v[hb + i];
     if (threadIdx.x == 0) s_abort = 0;

@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(kSesmStreamThreads, 1) k_persistent_sesm_strea
         h2[i] = x;
     }
     if (A.vcache) {
-        cache_incidences(P, smem_raw, v0, nown);
+        cache_incidences(P, smem_raw, v0, nown, threadIdx.x, T);
         for (int i = threadIdx.x; i < nown; i += T) s_inv[i] = P.inv_av[v0 + i];
         for (int i = threadIdx.x; i < nhalo; i += T) s_halo[i] = P.halo_v[hb + i];
     }

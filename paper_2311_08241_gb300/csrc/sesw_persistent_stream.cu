@@ -110,7 +110,7 @@ __device__ __forceinline__ void stream_patch(const SArgs &A, const int p, const 
     for (int i = threadIdx.x; i < nown; i += T) seta[i] = P.eta_in[v0 + i];
     for (int i = threadIdx.x; i < nhalo; i += T) seta[nown + i] = P.eta_in[P.halo_v[hb + i]];
     if (A.vcache) {
-        cache_incidences(P, smem_raw, v0, nown);
+        cache_incidences(P, smem_raw, v0, nown, threadIdx.x, T);
         for (int i = threadIdx.x; i < nown; i += T) s_inv[i] = P.inv_av[v0 + i];
         for (int i = threadIdx.x; i < nhalo; i += T) s_halo[i] = P.halo_v[hb + i];
     }
@@ -186,7 +186,7 @@ __device__ __forceinline__ void stream_patch(const SArgs &A, const int p, const 
             float e = vertex_eta(seta[i], sum, inv);
             if (EXTRA) {
                 if (P.W) e = __fmaf_rn(-dt, __ldg(P.W + v0 + i), e);
-                if (P.eta_sum) P.eta_sum[v0 + i] += seta[i];
+                if (P.eta_sum) P.eta_sum[v0 + i] = (m == 0 ? 0.0f : P.eta_sum[v0 + i]) + seta[i];
             }
             seta[i] = e;
             if (publish) st_relaxed_gpu_u64(xout + v0 + i, tag_out | __float_as_uint(e));
