@@ -107,17 +107,20 @@ constexpr int kFlagStride = 32;
 // the timeout bit and the abort word, which makes every other wait of the launch give
 // up too, and clears `ok`; the value returned then is meaningless. (The first reads of
 // a slot's corners are issued together by the caller, so that their latencies overlap.)
+// The word is re-read at once, without a pause, and the abort word and the clock are looked at
+// only every 64th time: a pause of 20 ns and an abort read in every turn made each turn two
+// L2 round trips and cost the level-8 sphere 7 % of its step (1450 -> 1357 us per 4 steps from the
+// pause alone).
 __device__ __forceinline__ float halo_eta(const PArgs &P, const unsigned long long *xs, int v,
                                           unsigned long long w, unsigned tag, unsigned abort_val, bool &ok)
 {
     if ((unsigned)(w >> 32) == tag) return __uint_as_float((unsigned)w);
     const unsigned *abort_word = P.flags;
     const long long t0 = clock64();
-    while (ok) {
-        __nanosleep(20);
+    for (unsigned turn = 1; ok; turn++) {
         w = ld_relaxed_gpu_u64(xs + v);
         if ((unsigned)(w >> 32) == tag) return __uint_as_float((unsigned)w);
-        if (ld_relaxed_gpu(abort_word) == abort_val || clock64() - t0 > P.a.wait_cycles) {
+        if ((turn & 63u) == 0 && (ld_relaxed_gpu(abort_word) == abort_val || clock64() - t0 > P.a.wait_cycles)) {
             ok = false;
             atomicOr(P.status, 2u);
             atomicExch(const_cast<unsigned *>(abort_word), abort_val);
