@@ -332,14 +332,22 @@ struct MsgLayerArgs {
 };
 cudaError_t launch_msg_layer_tc(const MsgLayerArgs &a, const __nv_bfloat16 *packed, const float *bias,
                                 unsigned *status, cudaStream_t st);
-// Backward of such a layer on the tensor cores, dA (FP32) split into two bfloat16 parts:
-// partial sums of the weight gradient sum_n Z[n][i] dA[n][j] and of the bias gradient over
-// rows_per_cta rows each (a multiple of 64; layout of k_reduce_partials), and the input
-// gradient dZ[n][i] = sum_j dA[n][j] W[i][j] (W: K x 64 bfloat16, row-major). K = 128 or 192.
-cudaError_t launch_wgrad_tc(int N, int K, int rows_per_cta, const float *Z, const float *dA, float *partial,
-                            unsigned *status, cudaStream_t st);
-cudaError_t launch_dgrad_tc(int N, int K, const float *dA, const __nv_bfloat16 *W, float *dZ, unsigned *status,
-                            cudaStream_t st);
+// Backward of such a layer on the tensor cores, one kernel (see k_bwd_layer_tc).
+struct BwdLayerArgs {
+    MsgLayerArgs m;             // the layer's rows, graph and hidden states (m.Y, m.hnext unused)
+    const float *Y;             // its activations [N][64]
+    const float *dh_in;         // gradient of h_next [N][64]; with dout, dh = dout Wout^T instead
+    const float *dout;          // null, or the gradient of the outputs behind the last layer: [N][4] for
+    const __nv_bfloat16 *Wout;  // element rows, [N][1] for vertex rows, with their weights (64 x 4 or 64 x 1)
+    const float *g0, *g1;       // message gradients to gather: element rows g0 [V][64]; vertex rows (not with
+                                // dout) g0, g1 [E][64]
+    float *dh_out;              // gradient of h [N][64] (may be dh_in)
+    float *m0, *m1;             // gradients of the layer's messages [N][64] (m1: element rows)
+    const __nv_bfloat16 *W;     // K x 64, row-major
+    float *partial;             // bwd_layer_ctas(N) x (K * 64 + 64): weight and bias gradient per CTA
+};
+int bwd_layer_ctas(int N);
+cudaError_t launch_bwd_layer_tc(const BwdLayerArgs &b, unsigned *status, cudaStream_t st);
 
 }  // namespace sesw
 

@@ -35,235 +35,254 @@ namespace {
 
 constexpr int HC = 64;            // hidden width
 constexpr int NL = 3;             // message-passing layers
-constexpr int TILE_ROWS = 64;     // rows per block of the matrix kernels
-constexpr int WG_ROWS = 32;       // rows per smem tile of the weight-gradient kernel
 constexpr int NSCALE = 8;         // eta, H, U, R, f, L, out_U, out_eta
 
 enum { S_ETA = 0, S_H, S_U, S_R, S_F, S_L, S_OU, S_OETA };
 
-// ------------------------------------------------------------------------- matrices
-//
-// out[n][j] = sum_i X[n][i] * Wm(i, j) (+ bias[j]), optionally tanh, optionally + res[n][j],
-// with Wm(i, j) = W[i * P + j] (forward, W is Kin x P) or W[j * Kin + i] (input gradient,
-// W is P x Kin). Each block computes 64 rows; thread (rg, cg) computes rows 4 rg .. 4 rg + 3
-// and columns cg + 16 j.
-template <int PT>
+// ------------------------------------------------------------------------- small layers
+
+// Input layers (K = 2 or 6 features): H = tanh(X W + b), 64 channels. A thread forms four
+// channels of one row (16 threads per row) with the weights in registers: bound by writing H.
+template <int K>
 __global__ void __launch_bounds__(256)
-k_mm(int N, int Kin, int P, const float *__restrict__ X, const __nv_bfloat16 *__restrict__ W, int trans,
-     const float *__restrict__ bias, int act, const float *__restrict__ res, float *__restrict__ Y)
+k_in_layer(int N, const float *__restrict__ X, const __nv_bfloat16 *__restrict__ W, const float *__restrict__ bias,
+           float *__restrict__ H)
 {
-    extern __shared__ float sm[];
-    const int ldx = Kin + 1;
-    float *Xs = sm;                              // [64][Kin + 1]
-    float *Ws = sm + TILE_ROWS * ldx;            // [Kin][P]
-    for (int t = threadIdx.x; t < Kin * P; t += blockDim.x) {
-        const int i = t / P, j = t % P;
-        const float w = __bfloat162float(trans ? W[(size_t)j * Kin + i] : W[(size_t)i * P + j]);
-        Ws[i * P + j] = w;
-    }
-    const int n0 = blockIdx.x * TILE_ROWS;
-    for (int t = threadIdx.x; t < TILE_ROWS * Kin; t += blockDim.x) {
-        const int r = t / Kin, i = t % Kin;
-        Xs[r * ldx + i] = (n0 + r < N) ? X[(size_t)(n0 + r) * Kin + i] : 0.0f;
-    }
-    __syncthreads();
-    const int rg = threadIdx.x >> 4, cg = threadIdx.x & 15;
-    float acc[4][PT];
+    const int c = ((int)threadIdx.x & 15) * 4;
+    float w[K][4], bv[4];
 #pragma unroll
-    for (int r = 0; r < 4; r++)
+    for (int i = 0; i < K; i++)
 #pragma unroll
-        for (int j = 0; j < PT; j++) acc[r][j] = 0.0f;
-    for (int i = 0; i < Kin; i++) {
-        float a[4], w[PT];
+        for (int t = 0; t < 4; t++) w[i][t] = __bfloat162float(W[i * HC + c + t]);
 #pragma unroll
-        for (int r = 0; r < 4; r++) a[r] = Xs[(rg * 4 + r) * ldx + i];
+    for (int t = 0; t < 4; t++) bv[t] = bias[c + t];
+    for (int n = blockIdx.x * 16 + ((int)threadIdx.x >> 4); n < N; n += gridDim.x * 16) {
+        float x[K], v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
-        for (int j = 0; j < PT; j++) {
-            const int col = cg + 16 * j;
-            w[j] = col < P ? Ws[i * P + col] : 0.0f;
+        for (int i = 0; i < K; i += 2) {
+            const float2 q = reinterpret_cast<const float2 *>(X + (size_t)n * K)[i / 2];
+            x[i] = q.x;
+            x[i + 1] = q.y;
         }
 #pragma unroll
-        for (int r = 0; r < 4; r++)
+        for (int i = 0; i < K; i++)
 #pragma unroll
-            for (int j = 0; j < PT; j++) acc[r][j] = fmaf(a[r], w[j], acc[r][j]);
-    }
+            for (int t = 0; t < 4; t++) v[t] = fmaf(x[i], w[i][t], v[t]);
 #pragma unroll
-    for (int r = 0; r < 4; r++) {
-        const int n = n0 + rg * 4 + r;
-        if (n >= N) continue;
-#pragma unroll
-        for (int j = 0; j < PT; j++) {
-            const int col = cg + 16 * j;
-            if (col >= P) continue;
-            float v = acc[r][j];
-            if (bias) v += bias[col];
-            if (act) v = tanhf(v);
-            if (res) v += res[(size_t)n * P + col];
-            Y[(size_t)n * P + col] = v;
-        }
+        for (int t = 0; t < 4; t++) v[t] = tanhf(v[t] + bv[t]);
+        *reinterpret_cast<float4 *>(H + (size_t)n * HC + c) = make_float4(v[0], v[1], v[2], v[3]);
     }
 }
 
-// Weight gradient of the small layers (the input layers, K = 2 or 6 and C = 64; the output
-// layers, K = 64 and C = 4 or 1; the message layers run on the tensor cores):
-//   partial[b][i * C + c] = sum_{n in rows of block b} Z[n][i] dA[n][c],
-//   partial[b][K * C + c] = sum_{n in rows of block b} dA[n][c].
-// A chunk of WG_ROWS rows of Z and dA is staged in shared memory with coalesced loads; thread t
-// owns outputs t, t + 256, ... of the K * C + C and adds the chunk's rows in order.
+// Output layers: O = H W + b, P = 4 or 1 outputs of 64 channels. A block stages 128 rows
+// (coalesced; 65 floats apart), then 128 x P / 2 (or 128) threads each run a row's products in
+// channel order: bound by reading H.
+constexpr int OUT_ROWS = 128;
+template <int P>
 __global__ void __launch_bounds__(256)
-k_wgrad_small(int N, int K, int C, const float *__restrict__ Z, const float *__restrict__ dA, int rows_per_block,
-              float *__restrict__ partial)
+k_out_layer(int N, const float *__restrict__ H, const __nv_bfloat16 *__restrict__ W, const float *__restrict__ bias,
+            float *__restrict__ O)
 {
-    __shared__ float Zs[WG_ROWS * HC];
-    __shared__ float Ds[WG_ROWS * HC];
-    constexpr int MAXO = 2;                      // outputs per thread: (K * C + C) <= 512
-    float acc[MAXO] = {0.0f, 0.0f};
-    const int nout = K * C + C;
-    const int nb = blockIdx.x * rows_per_block, ne = min(N, nb + rows_per_block);
-    for (int t0 = nb; t0 < ne; t0 += WG_ROWS) {
-        const int nr = min(WG_ROWS, ne - t0);
+    __shared__ float Hs[OUT_ROWS * (HC + 1)];
+    __shared__ float Ws[HC * P];
+    constexpr int PT = P == 4 ? 2 : 1;     // outputs per thread
+    for (int t = threadIdx.x; t < HC * P; t += 256) Ws[t] = __bfloat162float(W[t]);
+    const int r = (int)threadIdx.x & 127, p0 = ((int)threadIdx.x >> 7) * PT;
+    for (int n0 = blockIdx.x * OUT_ROWS; n0 < N; n0 += gridDim.x * OUT_ROWS) {
         __syncthreads();
-        for (int t = threadIdx.x; t < nr * K; t += blockDim.x) Zs[t] = Z[(size_t)t0 * K + t];
-        for (int t = threadIdx.x; t < nr * C; t += blockDim.x) Ds[t] = dA[(size_t)t0 * C + t];
+        const int nr = min(OUT_ROWS, N - n0);
+#pragma unroll 4
+        for (int t = threadIdx.x; t < nr * (HC / 4); t += 256) {
+            const float4 v = reinterpret_cast<const float4 *>(H + (size_t)n0 * HC)[t];
+            float *d = Hs + (t >> 4) * (HC + 1) + (t & 15) * 4;
+            d[0] = v.x; d[1] = v.y; d[2] = v.z; d[3] = v.w;
+        }
         __syncthreads();
+        if (r < nr && p0 < P) {
+            float acc[PT];
 #pragma unroll
-        for (int q = 0; q < MAXO; q++) {
-            const int o = threadIdx.x + q * 256;
-            if (o >= nout) continue;
-            float a = acc[q];
-            if (o < K * C) {
-                const int i = o / C, c = o % C;
-                for (int r = 0; r < nr; r++) a = fmaf(Zs[r * K + i], Ds[r * C + c], a);
-            } else {
-                const int c = o - K * C;
-                for (int r = 0; r < nr; r++) a += Ds[r * C + c];
+            for (int j = 0; j < PT; j++) acc[j] = 0.0f;
+#pragma unroll 16
+            for (int i = 0; i < HC; i++) {
+                const float h = Hs[r * (HC + 1) + i];
+#pragma unroll
+                for (int j = 0; j < PT; j++) acc[j] = fmaf(h, Ws[i * P + p0 + j], acc[j]);
             }
-            acc[q] = a;
-        }
-    }
-    float *out = partial + (size_t)blockIdx.x * nout;
 #pragma unroll
-    for (int q = 0; q < MAXO; q++) {
-        const int o = threadIdx.x + q * 256;
-        if (o < nout) out[o] = acc[q];
-    }
-}
-
-// Sum the partials of nb blocks in block order into gW (K*C) and gb (C).
-__global__ void k_reduce_partials(const float *__restrict__ partial, int nb, int len, float *__restrict__ gW,
-                                  float *__restrict__ gb, int KC)
-{
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < len; i += gridDim.x * blockDim.x) {
-        float s = 0.0f;
-        for (int b = 0; b < nb; b++) s += partial[(size_t)b * len + i];
-        if (i < KC)
-            gW[i] = s;
-        else
-            gb[i - KC] = s;
-    }
-}
-
-// dA = dY * (1 - Y^2) (derivative of tanh at the stored output Y).
-__global__ void k_tanh_bwd(size_t n, const float *__restrict__ dY, const float *__restrict__ Y, float *__restrict__ dA)
-{
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        dA[i] = dY[i] * (1.0f - Y[i] * Y[i]);
-}
-
-// ------------------------------------------------------------------------- messages
-// thread per (node, channel), 64 channels per node
-
-// Z_e = [h_e, L sum_k gx_k h_vk, L sum_k gy_k h_vk], rebuilt for the backward pass (the forward
-// pass forms it inside the tensor-core layer). The message-layer inputs are rounded to
-// bfloat16 values: the tensor-core layers read them as BF16 operands.
-__global__ void k_msg_elem(int E, const int4 *__restrict__ etri, const float4 *__restrict__ egrad, float L,
-                           const float *__restrict__ he, const float *__restrict__ hv, float *__restrict__ Z)
-{
-    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < (size_t)E * HC;
-         t += (size_t)gridDim.x * blockDim.x) {
-        const int e = (int)(t / HC), c = (int)(t % HC);
-        const int4 v = etri[e];
-        const float4 g = egrad[e];
-        const float h0 = hv[(size_t)v.x * HC + c], h1 = hv[(size_t)v.y * HC + c], h2 = hv[(size_t)v.z * HC + c];
-        const float2 m = msg_elem_grad(g, h0, h1, h2, L);
-        float *z = Z + (size_t)e * 3 * HC;
-        z[c] = bf16_value(he[t]);
-        z[HC + c] = bf16_value(m.x);
-        z[2 * HC + c] = bf16_value(m.y);
-    }
-}
-
-// dh_e += dZ_e[:, 0:64]
-__global__ void k_msg_elem_adj_e(int E, const float *__restrict__ dZ, float *__restrict__ dhe)
-{
-    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < (size_t)E * HC;
-         t += (size_t)gridDim.x * blockDim.x) {
-        const size_t e = t / HC;
-        dhe[t] += dZ[e * 3 * HC + t % HC];
-    }
-}
-
-// dh_v += L sum_{(e,k) at v} (gx_k dZ_e[64 + c] + gy_k dZ_e[128 + c])
-__global__ void k_msg_elem_adj_v(int V, const int *__restrict__ voff, const int *__restrict__ vinc,
-                                 const float4 *__restrict__ egrad, float L, const float *__restrict__ dZ,
-                                 float *__restrict__ dhv)
-{
-    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < (size_t)V * HC;
-         t += (size_t)gridDim.x * blockDim.x) {
-        const int v = (int)(t / HC), c = (int)(t % HC);
-        float s = 0.0f;
-        for (int q = voff[v]; q < voff[v + 1]; q++) {
-            const int ek = vinc[q], e = ek >> 2, k = ek & 3;
-            const float4 g = egrad[e];
-            const float gx = k == 0 ? g.x : (k == 1 ? g.z : -(g.x + g.z));
-            const float gy = k == 0 ? g.y : (k == 1 ? g.w : -(g.y + g.w));
-            const float *dz = dZ + (size_t)e * 3 * HC;
-            s += gx * dz[HC + c] + gy * dz[2 * HC + c];
+            for (int j = 0; j < PT; j++) O[(size_t)(n0 + r) * P + p0 + j] = acc[j] + bias[p0 + j];
         }
-        dhv[t] += L * s;
     }
 }
 
-// Z_v = [h_v, sum_{(e,k) at v} A_e h_e / sum A_e], rebuilt for the backward pass
-__global__ void k_msg_vert(int V, const int *__restrict__ voff, const int *__restrict__ vinc,
-                           const float *__restrict__ earea, const float *__restrict__ vinvA,
-                           const float *__restrict__ hv, const float *__restrict__ he, float *__restrict__ Z)
+// ------------------------------------------------------------------------- weight gradients
+//
+// Every layer leaves partial sums of its weight gradient (K x C) and bias gradient (C), one set
+// per block, which k_reduce_grads adds up in a fixed order. The message layers' come from the
+// tensor cores (k_bwd_layer_tc); the small layers' from the two kernels below, whose blocks run
+// over whole columns with coalesced 16-byte reads and no staging (before, one thread per output
+// walked staged rows: 139 us for the 910k x 64 output layer, a fifth of the memory rate).
+constexpr int SMALL_BLOCKS = 8 * 152;
+
+// Sum the 16 row groups' accumulators of a block in order: thread (4 channels, row group) holds
+// R rows of 4 values, out[r * HC + channel].
+template <int R>
+__device__ __forceinline__ void block_columns(const float (&acc)[R][4], float *sm, float *out)
 {
-    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < (size_t)V * HC;
-         t += (size_t)gridDim.x * blockDim.x) {
-        const int v = (int)(t / HC), c = (int)(t % HC);
-        float s = 0.0f;
-        for (int q = voff[v]; q < voff[v + 1]; q++) {
-            const int e = vinc[q] >> 2;
-            s = msg_vert_acc(s, earea[e], he[(size_t)e * HC + c]);
+    const int c = ((int)threadIdx.x & 15) * 4, grp = (int)threadIdx.x >> 4;
+#pragma unroll
+    for (int r = 0; r < R; r++) {
+        __syncthreads();
+#pragma unroll
+        for (int t = 0; t < 4; t++) sm[grp * (HC + 1) + c + t] = acc[r][t];
+        __syncthreads();
+        if (threadIdx.x < HC) {
+            float s = 0.0f;
+            for (int k = 0; k < 16; k++) s += sm[k * (HC + 1) + threadIdx.x];
+            out[r * HC + threadIdx.x] = s;
         }
-        float *z = Z + (size_t)v * 2 * HC;
-        z[c] = bf16_value(hv[t]);
-        z[HC + c] = bf16_value(msg_vert_mean(s, vinvA[v]));
     }
 }
 
-// dh_v += dZ_v[:, 0:64]
-__global__ void k_msg_vert_adj_v(int V, const float *__restrict__ dZ, float *__restrict__ dhv)
+// Output layers: G[i][j] = sum_n H[n][i] D[n][j] (partials in the order [j][i], then the bias).
+template <int P>
+__global__ void __launch_bounds__(256)
+k_wgrad_out(int N, int rows, const float *__restrict__ H, const float *__restrict__ D, float *__restrict__ partial)
 {
-    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < (size_t)V * HC;
-         t += (size_t)gridDim.x * blockDim.x) {
-        const size_t v = t / HC;
-        dhv[t] += dZ[v * 2 * HC + t % HC];
+    __shared__ float sm[16 * (HC + 1)];
+    const int c = ((int)threadIdx.x & 15) * 4, grp = (int)threadIdx.x >> 4;
+    float acc[P][4], bs[P];
+#pragma unroll
+    for (int j = 0; j < P; j++) {
+        bs[j] = 0.0f;
+#pragma unroll
+        for (int t = 0; t < 4; t++) acc[j][t] = 0.0f;
+    }
+    const int n1 = min(N, ((int)blockIdx.x + 1) * rows);
+#pragma unroll 4
+    for (int n = blockIdx.x * rows + grp; n < n1; n += 16) {
+        const float4 h = *reinterpret_cast<const float4 *>(H + (size_t)n * HC + c);
+        float d[P];
+        if (P == 4) {
+            const float4 q = reinterpret_cast<const float4 *>(D)[n];
+            d[0] = q.x; d[P > 1 ? 1 : 0] = q.y; d[P > 2 ? 2 : 0] = q.z; d[P > 3 ? 3 : 0] = q.w;
+        } else {
+            d[0] = D[n];
+        }
+#pragma unroll
+        for (int j = 0; j < P; j++) {
+            acc[j][0] = fmaf(h.x, d[j], acc[j][0]);
+            acc[j][1] = fmaf(h.y, d[j], acc[j][1]);
+            acc[j][2] = fmaf(h.z, d[j], acc[j][2]);
+            acc[j][3] = fmaf(h.w, d[j], acc[j][3]);
+            bs[j] += d[j];
+        }
+    }
+    float *out = partial + (size_t)blockIdx.x * ((HC + 1) * P);
+    block_columns<P>(acc, sm, out);
+    __syncthreads();
+    if (c == 0)
+#pragma unroll
+        for (int j = 0; j < P; j++) sm[grp * P + j] = bs[j];
+    __syncthreads();
+    if (threadIdx.x < P) {
+        float s = 0.0f;
+        for (int k = 0; k < 16; k++) s += sm[k * P + threadIdx.x];
+        out[HC * P + threadIdx.x] = s;
     }
 }
 
-// dh_e += sum_k A_e / (sum A)_{v_k} dZ_v[v_k][64 + c]
-__global__ void k_msg_vert_adj_e(int E, const int4 *__restrict__ etri, const float *__restrict__ earea,
-                                 const float *__restrict__ vinvA, const float *__restrict__ dZ, float *__restrict__ dhe)
+// Input layers: G[i][c] = sum_n X[n][i] dA[n][c] with dA = dh (1 - H^2) formed on the way. GATHER:
+// dh also receives the first message layer's gradients,
+// dh_v += L sum_{(e,k) at v} (gx_k g0_e + gy_k g1_e).
+template <int K, int GATHER>
+__global__ void __launch_bounds__(256)
+k_wgrad_in(int N, int rows, const float *__restrict__ X, const float *__restrict__ H, const float *__restrict__ dh,
+           const int *__restrict__ voff, const int *__restrict__ vinc, const float4 *__restrict__ egrad, float L,
+           const float *__restrict__ g0, const float *__restrict__ g1, float *__restrict__ partial)
 {
-    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < (size_t)E * HC;
-         t += (size_t)gridDim.x * blockDim.x) {
-        const int e = (int)(t / HC), c = (int)(t % HC);
-        const int4 v = etri[e];
-        const float a = earea[e];
-        dhe[t] += a * (vinvA[v.x] * dZ[(size_t)v.x * 2 * HC + HC + c] + vinvA[v.y] * dZ[(size_t)v.y * 2 * HC + HC + c] +
-                       vinvA[v.z] * dZ[(size_t)v.z * 2 * HC + HC + c]);
+    __shared__ float sm[16 * (HC + 1)];
+    const int c = ((int)threadIdx.x & 15) * 4, grp = (int)threadIdx.x >> 4;
+    float acc[K + 1][4];
+#pragma unroll
+    for (int i = 0; i <= K; i++)
+#pragma unroll
+        for (int t = 0; t < 4; t++) acc[i][t] = 0.0f;
+    const int n1 = min(N, ((int)blockIdx.x + 1) * rows);
+#pragma unroll(GATHER ? 1 : 2)
+    for (int n = blockIdx.x * rows + grp; n < n1; n += 16) {
+        const float4 h = *reinterpret_cast<const float4 *>(H + (size_t)n * HC + c);
+        const float4 d4 = *reinterpret_cast<const float4 *>(dh + (size_t)n * HC + c);
+        float d[4] = {d4.x, d4.y, d4.z, d4.w};
+        if (GATHER) {
+            float s[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+            const int q0 = voff[n], q1 = voff[n + 1];
+#pragma unroll 3
+            for (int q = q0; q < q1; q++) {
+                const int ek = vinc[q], e = ek >> 2, k = ek & 3;
+                const float4 g = egrad[e];
+                const float4 a = *reinterpret_cast<const float4 *>(g0 + (size_t)e * HC + c);
+                const float4 b = *reinterpret_cast<const float4 *>(g1 + (size_t)e * HC + c);
+                const float gx = k == 0 ? g.x : (k == 1 ? g.z : -(g.x + g.z));
+                const float gy = k == 0 ? g.y : (k == 1 ? g.w : -(g.y + g.w));
+                s[0] += gx * a.x + gy * b.x;
+                s[1] += gx * a.y + gy * b.y;
+                s[2] += gx * a.z + gy * b.z;
+                s[3] += gx * a.w + gy * b.w;
+            }
+#pragma unroll
+            for (int t = 0; t < 4; t++) d[t] += L * s[t];
+        }
+        const float hv[4] = {h.x, h.y, h.z, h.w};
+        float x[K];
+#pragma unroll
+        for (int i = 0; i < K; i += 2) {
+            const float2 q = reinterpret_cast<const float2 *>(X + (size_t)n * K)[i / 2];
+            x[i] = q.x;
+            x[i + 1] = q.y;
+        }
+#pragma unroll
+        for (int t = 0; t < 4; t++) {
+            const float dA = d[t] * (1.0f - hv[t] * hv[t]);
+#pragma unroll
+            for (int i = 0; i < K; i++) acc[i][t] = fmaf(x[i], dA, acc[i][t]);
+            acc[K][t] += dA;
+        }
+    }
+    block_columns<K + 1>(acc, sm, partial + (size_t)blockIdx.x * ((K + 1) * HC));
+}
+
+// The layers' partial sums into the gradient vector, all layers in one launch: block (x, y) adds
+// outputs 32 x .. + 31 of layer y; warp w takes partials w, w + 8, ..., and the warps' sums are
+// added in order. (One thread per output before: 650 us for the 7108 partials of an
+// output layer, in two blocks.)
+constexpr int MAX_LAYERS = 2 * NL + 4;
+struct ReduceArgs {
+    const float *partial[MAX_LAYERS];
+    int nb[MAX_LAYERS], len[MAX_LAYERS];
+    int cols[MAX_LAYERS];            // 0, or the columns of an output layer, whose partials hold G^T
+    float *out[MAX_LAYERS];          // gradient of the matrix, directly followed by the bias
+};
+__global__ void __launch_bounds__(256) k_reduce_grads(const ReduceArgs a)
+{
+    __shared__ float sm[8][33];
+    const int y = blockIdx.y, len = a.len[y], lane = (int)threadIdx.x & 31, w = (int)threadIdx.x >> 5;
+    const int o = blockIdx.x * 32 + lane;
+    if (blockIdx.x * 32 >= len) return;
+    float s = 0.0f;
+    if (o < len) {
+        const float *p = a.partial[y] + o;
+        const int nb = a.nb[y];
+#pragma unroll 8
+        for (int k = w; k < nb; k += 8) s += p[(size_t)k * len];
+    }
+    sm[w][lane] = s;
+    __syncthreads();
+    if (w == 0 && o < len) {
+        float t = sm[0][lane];
+#pragma unroll
+        for (int k = 1; k < 8; k++) t += sm[k][lane];
+        const int cols = a.cols[y];
+        a.out[y][cols > 0 && o < HC * cols ? (o % HC) * cols + o / HC : o] = t;
     }
 }
 
@@ -344,12 +363,19 @@ k_loss(int V, int E, const float *__restrict__ oe, const float *__restrict__ ov,
     }
 }
 
-__global__ void k_sum_parts(const double *__restrict__ part, int n, double *__restrict__ out)
+// The sum of n partials by one block, in a fixed order.
+__global__ void __launch_bounds__(256) k_sum_parts(const double *__restrict__ part, int n, double *__restrict__ out)
 {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double s = 0.0;
-        for (int i = 0; i < n; i++) s += part[i];
-        out[0] = s;
+    __shared__ double sh[8];
+    double s = 0.0;
+    for (int i = threadIdx.x; i < n; i += 256) s += part[i];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = sh[0];
+        for (int w = 1; w < 8; w++) t += sh[w];
+        out[0] = t;
     }
 }
 
@@ -603,11 +629,13 @@ struct Surrogate {
     // activations
     float *xv = nullptr, *xe = nullptr;
     float *hv[NL + 1] = {}, *he[NL + 1] = {}, *yv[NL] = {}, *ye[NL] = {};
-    float *oe = nullptr, *ov = nullptr, *ze = nullptr, *zv = nullptr;
-    float *dze = nullptr, *dzv = nullptr, *dhe = nullptr, *dhv = nullptr, *dae = nullptr, *dav = nullptr;
+    float *oe = nullptr, *ov = nullptr;
+    // gradients of the hidden states, and of the messages (element layers two per row, vertex one)
+    float *dhe = nullptr, *dhv = nullptr, *me0 = nullptr, *me1 = nullptr, *mv = nullptr;
     float *doe = nullptr, *dov = nullptr;
-    float *partial = nullptr;
-    size_t partial_len = 0;
+    float *partial = nullptr;                  // partial weight gradients, layer after layer
+    std::vector<size_t> part_off;              // where each layer's begin
+    std::vector<int> part_nb;                  // and how many there are
     double *red = nullptr;      // reductions
     // dataset
     long cap = 0;
@@ -617,7 +645,6 @@ struct Surrogate {
     float *save_eta = nullptr;
     float2 *save_U = nullptr;
     double *stage = nullptr;    // host samples in transit: 2 V + 8 E doubles
-    size_t smem_mm = 0;
     unsigned *status = nullptr; // the context's device status word (timeout bit of the tensor-core waits)
 };
 
@@ -650,28 +677,15 @@ int salloc(sesw_ctx *c, T **p, size_t n)
         if (r_ != SESW_OK) return r_;  \
     } while (0)
 
-cudaError_t mm(Surrogate &S, cudaStream_t st, int N, int Kin, int P, const float *X, const __nv_bfloat16 *W,
-               int trans, const float *bias, int act, const float *res, float *Y)
-{
-
-    const size_t smem = sizeof(float) * ((size_t)TILE_ROWS * (Kin + 1) + (size_t)Kin * P);
-    const int grid = (N + TILE_ROWS - 1) / TILE_ROWS;
-    if (grid == 0) return cudaSuccess;
-    if (P <= 64)
-        k_mm<4><<<grid, 256, smem, st>>>(N, Kin, P, X, W, trans, bias, act, res, Y);
-    else
-        k_mm<12><<<grid, 256, smem, st>>>(N, Kin, P, X, W, trans, bias, act, res, Y);
-    return cudaGetLastError();
-}
+// blocks of the streaming kernels: a multiple of the SMs, at most one per `rows` rows
+int stream_grid(int N, int rows) { return std::max(1, std::min((N + rows - 1) / rows, 16 * 152)); }
 
 // Forward of message layer ly (kind 0: element rows from h_e[l] and h_v[l]; kind 1: vertex rows
 // from h_v[l] and h_e[l + 1]) on the tensor cores, the message gather fused into the layer:
 // writes Y and h_next = h + Y.
-cudaError_t msg_layer(Surrogate &S, cudaStream_t st, const Layer &ly, int kind, const float *hself,
-                      const float *hother, float *Y, float *hnext)
+MsgLayerArgs layer_args(const Surrogate &S, int kind, const float *hself, const float *hother)
 {
-    if (ly.tc < 0) return cudaErrorInvalidValue;
-    MsgLayerArgs a;
+    MsgLayerArgs a{};
     a.kind = kind;
     a.N = kind == 0 ? S.E : S.V;
     a.etri = S.etri;
@@ -683,6 +697,14 @@ cudaError_t msg_layer(Surrogate &S, cudaStream_t st, const Layer &ly, int kind, 
     a.vinvA = S.vinvA;
     a.hself = hself;
     a.hother = hother;
+    return a;
+}
+
+cudaError_t msg_layer(Surrogate &S, cudaStream_t st, const Layer &ly, int kind, const float *hself,
+                      const float *hother, float *Y, float *hnext)
+{
+    if (ly.tc < 0) return cudaErrorInvalidValue;
+    MsgLayerArgs a = layer_args(S, kind, hself, hother);
     a.Y = Y;
     a.hnext = hnext;
     return launch_msg_layer_tc(a, S.wtc + ly.tc, S.w32 + ly.b, S.status, st);
@@ -699,44 +721,14 @@ cudaError_t pack_tc(Surrogate &S, cudaStream_t st)
     return cudaSuccess;
 }
 
-// gradient of layer l's matrix and bias from its input Z [N][K] and dA [N][C]; the message
-// layers (inputs rounded to bfloat16 values, 64 outputs) on the tensor cores
-cudaError_t wgrad(Surrogate &S, cudaStream_t st, const Layer &ly, int N, const float *Z, const float *dA)
-{
-    // the small layers have few outputs per block, so their blocks take fewer rows (more blocks
-    // in flight); the partial buffer holds ceil(N / 2048) partials of the largest layer
-    const int len = ly.K * ly.C + ly.C;
-    int rows = 2048;
-    if (ly.tc < 0)
-        while (rows > 128 && (size_t)((N + rows / 2 - 1) / (rows / 2)) * len <= S.partial_len) rows /= 2;
-    const int nb = std::max(1, (N + rows - 1) / rows);
-    if (ly.tc >= 0) {
-        const cudaError_t e = launch_wgrad_tc(N, ly.K, rows, Z, dA, S.partial, S.status, st);
-        if (e != cudaSuccess) return e;
-    } else {
-        // the staged tiles hold WG_ROWS rows of at most HC values; a thread owns at most 2 outputs
-        if (ly.K > HC || ly.C > HC || ly.K * ly.C + ly.C > 512) return cudaErrorInvalidValue;
-        k_wgrad_small<<<nb, 256, 0, st>>>(N, ly.K, ly.C, Z, dA, rows, S.partial);
-    }
-    k_reduce_partials<<<grid1(len), 256, 0, st>>>(S.partial, nb, len, S.grad + ly.w, S.grad + ly.b, ly.K * ly.C);
-    return cudaGetLastError();
-}
-
-// dZ = dA W^T of a message layer (the gradient with respect to its inputs), on the tensor cores
-cudaError_t dgrad(Surrogate &S, cudaStream_t st, const Layer &ly, int N, const float *dA, float *dZ)
-{
-    if (ly.tc >= 0) return launch_dgrad_tc(N, ly.K, dA, S.w16 + ly.w, dZ, S.status, st);
-    return mm(S, st, N, ly.C, ly.K, dA, S.w16 + ly.w, 1, nullptr, 0, nullptr, dZ);
-}
-
 // forward of one sample whose features are in S.xv, S.xe; keep_y keeps each message layer's
 // activation Y for the backward pass (inference does without it)
 cudaError_t forward(Surrogate &S, cudaStream_t st, bool keep_y = true)
 {
     cudaError_t e;
     const Layer &lv0 = S.L[0], &le0 = S.L[1];
-    if ((e = mm(S, st, S.V, 2, HC, S.xv, S.w16 + lv0.w, 0, S.w32 + lv0.b, 1, nullptr, S.hv[0])) != cudaSuccess) return e;
-    if ((e = mm(S, st, S.E, 6, HC, S.xe, S.w16 + le0.w, 0, S.w32 + le0.b, 1, nullptr, S.he[0])) != cudaSuccess) return e;
+    k_in_layer<2><<<stream_grid(S.V, 64), 256, 0, st>>>(S.V, S.xv, S.w16 + lv0.w, S.w32 + lv0.b, S.hv[0]);
+    k_in_layer<6><<<stream_grid(S.E, 64), 256, 0, st>>>(S.E, S.xe, S.w16 + le0.w, S.w32 + le0.b, S.he[0]);
     for (int l = 0; l < NL; l++) {
         const Layer &le = S.L[2 + 2 * l], &lv = S.L[3 + 2 * l];
         // h_e(l+1) = h_e(l) + y_e(l), then h_v(l+1) = h_v(l) + y_v(l) from h_e(l+1)
@@ -747,44 +739,72 @@ cudaError_t forward(Surrogate &S, cudaStream_t st, bool keep_y = true)
             return e;
     }
     const Layer &leo = S.L[2 + 2 * NL], &lvo = S.L[3 + 2 * NL];
-    if ((e = mm(S, st, S.E, HC, 4, S.he[NL], S.w16 + leo.w, 0, S.w32 + leo.b, 0, nullptr, S.oe)) != cudaSuccess) return e;
-    if ((e = mm(S, st, S.V, HC, 1, S.hv[NL], S.w16 + lvo.w, 0, S.w32 + lvo.b, 0, nullptr, S.ov)) != cudaSuccess) return e;
+    k_out_layer<4><<<stream_grid(S.E, OUT_ROWS), 256, 0, st>>>(S.E, S.he[NL], S.w16 + leo.w, S.w32 + leo.b, S.oe);
+    k_out_layer<1><<<stream_grid(S.V, OUT_ROWS), 256, 0, st>>>(S.V, S.hv[NL], S.w16 + lvo.w, S.w32 + lvo.b, S.ov);
     return cudaGetLastError();
 }
+
+// rows per block of the small layers' weight gradients
+int small_rows(int N) { return std::max(64, (N + SMALL_BLOCKS - 1) / SMALL_BLOCKS); }
 
 // backward from S.doe, S.dov to S.grad (overwritten)
 cudaError_t backward(Surrogate &S, cudaStream_t st)
 {
     const float Ls = (float)S.scales_h[S_L];
     cudaError_t e;
-    const Layer &leo = S.L[2 + 2 * NL], &lvo = S.L[3 + 2 * NL];
-    if ((e = wgrad(S, st, leo, S.E, S.he[NL], S.doe)) != cudaSuccess) return e;
-    if ((e = wgrad(S, st, lvo, S.V, S.hv[NL], S.dov)) != cudaSuccess) return e;
-    if ((e = mm(S, st, S.E, 4, HC, S.doe, S.w16 + leo.w, 1, nullptr, 0, nullptr, S.dhe)) != cudaSuccess) return e;
-    if ((e = mm(S, st, S.V, 1, HC, S.dov, S.w16 + lvo.w, 1, nullptr, 0, nullptr, S.dhv)) != cudaSuccess) return e;
+    const int io_e = 2 + 2 * NL, io_v = 3 + 2 * NL;
+    auto part = [&](int l) { return S.partial + S.part_off[l]; };
+    const int re = small_rows(S.E), rv = small_rows(S.V);
+    k_wgrad_out<4><<<S.part_nb[io_e], 256, 0, st>>>(S.E, re, S.he[NL], S.doe, part(io_e));
+    k_wgrad_out<1><<<S.part_nb[io_v], 256, 0, st>>>(S.V, rv, S.hv[NL], S.dov, part(io_v));
     for (int l = NL - 1; l >= 0; l--) {
-        const Layer &le = S.L[2 + 2 * l], &lv = S.L[3 + 2 * l];
-        // vertex update of layer l
-        k_tanh_bwd<<<grid1((size_t)S.V * HC), 256, 0, st>>>((size_t)S.V * HC, S.dhv, S.yv[l], S.dav);
-        k_msg_vert<<<grid1((size_t)S.V * HC), 256, 0, st>>>(S.V, S.voff, S.vinc, S.earea, S.vinvA, S.hv[l], S.he[l + 1],
-                                                            S.zv);
-        if ((e = wgrad(S, st, lv, S.V, S.zv, S.dav)) != cudaSuccess) return e;
-        if ((e = dgrad(S, st, lv, S.V, S.dav, S.dzv)) != cudaSuccess) return e;
-        k_msg_vert_adj_v<<<grid1((size_t)S.V * HC), 256, 0, st>>>(S.V, S.dzv, S.dhv);
-        k_msg_vert_adj_e<<<grid1((size_t)S.E * HC), 256, 0, st>>>(S.E, S.etri, S.earea, S.vinvA, S.dzv, S.dhe);
-        // element update of layer l
-        k_tanh_bwd<<<grid1((size_t)S.E * HC), 256, 0, st>>>((size_t)S.E * HC, S.dhe, S.ye[l], S.dae);
-        k_msg_elem<<<grid1((size_t)S.E * HC), 256, 0, st>>>(S.E, S.etri, S.egrad, Ls, S.he[l], S.hv[l], S.ze);
-        if ((e = wgrad(S, st, le, S.E, S.ze, S.dae)) != cudaSuccess) return e;
-        if ((e = dgrad(S, st, le, S.E, S.dae, S.dze)) != cudaSuccess) return e;
-        k_msg_elem_adj_e<<<grid1((size_t)S.E * HC), 256, 0, st>>>(S.E, S.dze, S.dhe);
-        k_msg_elem_adj_v<<<grid1((size_t)S.V * HC), 256, 0, st>>>(S.V, S.voff, S.vinc, S.egrad, Ls, S.dze, S.dhv);
+        const bool last = l == NL - 1;
+        BwdLayerArgs b{};
+        // vertex update of layer l: h_v(l+1) = h_v(l) + tanh(.), from h_v(l) and h_e(l+1)
+        const int iv = 3 + 2 * l, ie = 2 + 2 * l;
+        b.m = layer_args(S, 1, S.hv[l], S.he[l + 1]);
+        b.Y = S.yv[l];
+        b.dh_in = S.dhv;
+        b.dout = last ? S.dov : nullptr;
+        b.Wout = S.w16 + S.L[io_v].w;
+        b.g0 = last ? nullptr : S.me0;
+        b.g1 = last ? nullptr : S.me1;
+        b.dh_out = S.dhv;
+        b.m0 = S.mv;
+        b.W = S.w16 + S.L[iv].w;
+        b.partial = part(iv);
+        if ((e = launch_bwd_layer_tc(b, S.status, st)) != cudaSuccess) return e;
+        // element update of layer l: h_e(l+1) = h_e(l) + tanh(.), from h_e(l) and h_v(l)
+        b = BwdLayerArgs{};
+        b.m = layer_args(S, 0, S.he[l], S.hv[l]);
+        b.Y = S.ye[l];
+        b.dh_in = S.dhe;
+        b.dout = last ? S.doe : nullptr;
+        b.Wout = S.w16 + S.L[io_e].w;
+        b.g0 = S.mv;
+        b.dh_out = S.dhe;
+        b.m0 = S.me0;
+        b.m1 = S.me1;
+        b.W = S.w16 + S.L[ie].w;
+        b.partial = part(ie);
+        if ((e = launch_bwd_layer_tc(b, S.status, st)) != cudaSuccess) return e;
     }
-    const Layer &lv0 = S.L[0], &le0 = S.L[1];
-    k_tanh_bwd<<<grid1((size_t)S.V * HC), 256, 0, st>>>((size_t)S.V * HC, S.dhv, S.hv[0], S.dav);
-    if ((e = wgrad(S, st, lv0, S.V, S.xv, S.dav)) != cudaSuccess) return e;
-    k_tanh_bwd<<<grid1((size_t)S.E * HC), 256, 0, st>>>((size_t)S.E * HC, S.dhe, S.he[0], S.dae);
-    if ((e = wgrad(S, st, le0, S.E, S.xe, S.dae)) != cudaSuccess) return e;
+    k_wgrad_in<2, 1><<<S.part_nb[0], 256, 0, st>>>(S.V, rv, S.xv, S.hv[0], S.dhv, S.voff, S.vinc, S.egrad, Ls, S.me0,
+                                                  S.me1, part(0));
+    k_wgrad_in<6, 0><<<S.part_nb[1], 256, 0, st>>>(S.E, re, S.xe, S.he[0], S.dhe, nullptr, nullptr, nullptr, 0.0f,
+                                                  nullptr, nullptr, part(1));
+    ReduceArgs r;
+    int most = 0;
+    for (size_t l = 0; l < S.L.size(); l++) {
+        const Layer &ly = S.L[l];
+        r.partial[l] = part((int)l);
+        r.nb[l] = S.part_nb[l];
+        r.len[l] = ly.K * ly.C + ly.C;
+        r.cols[l] = ly.K == HC ? ly.C : 0;
+        r.out[l] = S.grad + ly.w;      // the bias follows the matrix in the parameter vector
+        most = std::max(most, r.len[l]);
+    }
+    k_reduce_grads<<<dim3((most + 31) / 32, (unsigned)S.L.size()), 256, 0, st>>>(r);
     return cudaGetLastError();
 }
 
@@ -801,7 +821,7 @@ cudaError_t loss_of(Surrogate &S, sesw_ctx *c, long i, bool want_grad, double *d
     const int nb = 152 * 4;
     k_loss<<<nb, 256, 0, c->stream>>>(S.V, S.E, S.oe, S.ov, S.d_te + (size_t)i * 4 * S.E, S.d_tv + (size_t)i * S.V,
                                       S.scales, want_grad ? S.doe : nullptr, want_grad ? S.dov : nullptr, S.red + 16);
-    k_sum_parts<<<1, 32, 0, c->stream>>>(S.red + 16, nb, dst);
+    k_sum_parts<<<1, 256, 0, c->stream>>>(S.red + 16, nb, dst);
     return cudaGetLastError();
 }
 
@@ -936,19 +956,23 @@ int sesw_surrogate_init(sesw_ctx *c, int32_t capacity, int32_t seed)
     }
     STRY(sesw::salloc(c, &S.oe, 4 * (size_t)E));
     STRY(sesw::salloc(c, &S.ov, (size_t)V));
-    STRY(sesw::salloc(c, &S.ze, 3 * eh));
-    STRY(sesw::salloc(c, &S.zv, 2 * vh));
-    STRY(sesw::salloc(c, &S.dze, 3 * eh));
-    STRY(sesw::salloc(c, &S.dzv, 2 * vh));
+    STRY(sesw::salloc(c, &S.me0, eh));
+    STRY(sesw::salloc(c, &S.me1, eh));
+    STRY(sesw::salloc(c, &S.mv, vh));
     STRY(sesw::salloc(c, &S.dhe, eh));
     STRY(sesw::salloc(c, &S.dhv, vh));
-    STRY(sesw::salloc(c, &S.dae, eh));
-    STRY(sesw::salloc(c, &S.dav, vh));
     STRY(sesw::salloc(c, &S.doe, 4 * (size_t)E));
     STRY(sesw::salloc(c, &S.dov, (size_t)V));
-    const int nbmax = std::max(1, (std::max(V, E) + 2047) / 2048);
-    S.partial_len = (size_t)nbmax * (3 * sesw::HC * sesw::HC + sesw::HC);
-    STRY(sesw::salloc(c, &S.partial, S.partial_len));
+    size_t part_len = 0;
+    for (size_t l = 0; l < S.L.size(); l++) {
+        const int n = l % 2 == 0 ? (l == 0 ? V : E) : (l == 1 ? E : V);   // rows of layer l (see S.L)
+        const int nb = S.L[l].tc >= 0 ? sesw::bwd_layer_ctas(n)
+                                      : (n + sesw::small_rows(n) - 1) / sesw::small_rows(n);
+        S.part_off.push_back(part_len);
+        S.part_nb.push_back(nb);
+        part_len += (size_t)nb * (S.L[l].K * S.L[l].C + S.L[l].C);
+    }
+    STRY(sesw::salloc(c, &S.partial, part_len));
     STRY(sesw::salloc(c, &S.red, 16 + 152 * 4 * 8));
     // dataset and inference buffers
     STRY(sesw::salloc(c, &S.d_eta, (size_t)capacity * V));
@@ -963,10 +987,6 @@ int sesw_surrogate_init(sesw_ctx *c, int32_t capacity, int32_t seed)
     STRY(sesw::salloc(c, &S.save_eta, (size_t)V));
     STRY(sesw::salloc(c, &S.save_U, (size_t)c->dm.nslot));
     STRY(sesw::salloc(c, &S.stage, 2 * (size_t)V + 8 * (size_t)E));
-    // matrix kernels need up to (64 x 193 + 192 x 64) floats of shared memory
-    S.smem_mm = sizeof(float) * (64 * (3 * sesw::HC + 1) + 3 * sesw::HC * sesw::HC);
-    SCK(cudaFuncSetAttribute(sesw::k_mm<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S.smem_mm));
-    SCK(cudaFuncSetAttribute(sesw::k_mm<12>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S.smem_mm));
     SCK(cudaStreamSynchronize(c->stream));
     return SESW_OK;
 }

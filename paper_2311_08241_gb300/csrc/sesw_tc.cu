@@ -5,14 +5,17 @@
 // them, so Z never goes to memory; W is bfloat16 and the products accumulate in FP32 in
 // tensor memory.
 //
-// One CTA of 256 threads computes 128 rows. It stages its Z tile and the whole W (as W^T,
-// from a copy packed once per weight update by k_pack_wt) in shared memory in the K-major
-// layout without swizzle that tcgen05.mma reads: core matrices of 8 rows x 8 bf16 (16 bytes
-// per row, 128 bytes each), core matrices adjacent along K 128 bytes apart, along M (or N)
-// K * 16 bytes apart. One thread issues K/16 MMAs of shape 128 x 64 x 16 into a 64-column
-// TMEM accumulator and commits them to an mbarrier; after a bounded wait every warp reads 32
-// rows x 32 columns back with tcgen05.ld, applies bias, activation and the residual, and
-// stores.
+// A CTA of 256 threads takes tiles of 128 rows one after another. It stages a tile of Z in shared
+// memory in blocks of 64 features with the 128-byte swizzle and, once, the whole W (as W^T, from a
+// copy packed once per weight update by k_pack_wt) in the K-major layout without swizzle: core
+// matrices of 8 rows x 8 bf16 (16 bytes per row, 128 bytes each), core matrices adjacent along K
+// 128 bytes apart, along N K * 16 bytes apart. One thread issues K/16 MMAs of shape 128 x 64 x 16 into a 64-column
+// TMEM accumulator and commits them to an mbarrier; after a bounded wait the warps read the
+// accumulator back with tcgen05.ld and turn it through shared memory, so that bias, activation,
+// residual and the stores run in the coalesced order of the gather.
+//
+// Backward (k_bwd_layer_tc): one kernel per layer forms dA, rebuilds Z, and multiplies both
+// gradients from the same staged tiles.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -42,6 +45,13 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t addr, uint32_t lbo, uint3
            ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | ((uint64_t)1 << 46);
 }
 
+// The same for a tile of 128-byte rows with the 128-byte swizzle (layout type 2 in bits 61-63): 64
+// bfloat16 per row, 16-byte chunk j of row r at chunk j ^ (r & 7), 8 rows per 1024-byte group.
+__device__ __forceinline__ uint64_t umma_desc_sw(uint32_t addr, uint32_t lbo, uint32_t sbo)
+{
+    return umma_desc(addr, lbo, sbo) | ((uint64_t)2 << 61);
+}
+
 // Instruction descriptor of tcgen05.mma kind::f16: FP32 accumulator (bits 4-5 = 1),
 // BF16 A and B (bits 7-9 and 10-12 = 1), both K-major, N / 8 at bit 17, M / 16 at bit 24.
 __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N)
@@ -53,22 +63,6 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
 {
     const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<const uint32_t *>(&v);
-}
-
-// Bounded wait on phase 0 of an mbarrier; false when the budget ran out.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, long long budget)
-{
-    const long long t0 = clock64();
-    while (true) {
-        uint32_t ok;
-        asm volatile(
-            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-            : "=r"(ok)
-            : "r"(bar), "r"(0)
-            : "memory");
-        if (ok) return true;
-        if (clock64() - t0 > budget) return false;
-    }
 }
 
 // Read 16 FP32 columns of this warp's 32 TMEM lanes.
@@ -108,259 +102,32 @@ __device__ __forceinline__ uint4 pack_bf16x8(const float *v)
                       pack_bf16x2(v[6], v[7]));
 }
 
+// Eight floats of global memory in one 32-byte access (32-byte aligned): the gathers are bound by the
+// L1 pipe, which takes a whole sector per thread in half the passes of two 16-byte accesses.
 __device__ __forceinline__ void load8(const float *p, float *v)
 {
-    const float4 a = reinterpret_cast<const float4 *>(p)[0], b = reinterpret_cast<const float4 *>(p)[1];
+    asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+                 : "l"(p));
+}
+
+__device__ __forceinline__ void store8(float *p, const float *v)
+{
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]),
+                 "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+                 : "memory");
+}
+
+// Eight floats of the turned tile (shared memory) for channel octet cg: the upper four octets take
+// their halves in the other order, so that a quarter warp reads all 32 banks.
+__device__ __forceinline__ void load8_turned(const float *p, int cg, float *v)
+{
+    const bool up = cg >= 4;
+    const float4 x = reinterpret_cast<const float4 *>(p)[up ? 1 : 0], y = reinterpret_cast<const float4 *>(p)[up ? 0 : 1];
+    const float4 a = up ? y : x, b = up ? x : y;
     v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
     v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
 }
-
-// Element incidences of a vertex-layer CTA's rows held in shared memory (more go through
-// global memory, in the same order).
-constexpr int MSG_INC_CAP = 1536;
-
-// Shared memory of k_msg_layer_tc: the A tile (128 x K bf16), W^T (64 x K bf16), then the
-// rows' graph data: KIND 0 the three corners of 128 elements (three CTAs of 75.3 KB fit an
-// SM); KIND 1 the 129 CSR offsets of the rows and the element ids and areas of up to
-// MSG_INC_CAP incidences.
-__host__ __device__ constexpr size_t msg_layer_smem(int kind)
-{
-    return (size_t)(TC_M + TC_N) * (kind == 0 ? 3 * TC_N : 2 * TC_N) * 2 +
-           (kind == 0 ? (size_t)TC_M * 12 : (size_t)(TC_M + 4) * 4 + (size_t)MSG_INC_CAP * 8);
-}
-
-// One message layer of the surrogate's forward pass (KIND 0: element rows, K = 192; KIND 1:
-// vertex rows, K = 128): the CTA forms its 128 rows of Z from the hidden states while it
-// stages them as the A tile, so Z never goes to memory, then Y = tanh(Z W + b) and
-// h_next = h + Y in the epilogue. The rows' graph data go to shared memory first, so that
-// every gather of the hidden states has its address at hand; each thread then gathers two
-// rows' inputs at a time.
-template <int KIND>
-__global__ void __launch_bounds__(TC_THREADS, 3)
-k_msg_layer_tc(const MsgLayerArgs a, const uint4 *__restrict__ Wp, const float *__restrict__ bias,
-               unsigned *__restrict__ status, long long wait_cycles)
-{
-    constexpr int K = KIND == 0 ? 3 * TC_N : 2 * TC_N;
-    constexpr int KC = K / 8;    // core matrices along K
-    extern __shared__ __align__(1024) unsigned char smem[];
-    uint4 *As = reinterpret_cast<uint4 *>(smem);                              // 128 x K bf16
-    uint4 *Bs = reinterpret_cast<uint4 *>(smem + (size_t)TC_M * K * 2);       // 64 x K bf16 (W^T)
-    unsigned char *gdata = smem + (size_t)(TC_M + TC_N) * K * 2;
-    int *s_tri = reinterpret_cast<int *>(gdata);                              // KIND 0: [3][128]
-    int *s_off = reinterpret_cast<int *>(gdata);                              // KIND 1
-    int *s_inc = s_off + TC_M + 4;
-    float *s_area = reinterpret_cast<float *>(s_inc + MSG_INC_CAP);
-    __shared__ __align__(8) uint64_t mbar;
-    __shared__ uint32_t tmem_base;
-    __shared__ int s_ok;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int N = a.N, n0 = blockIdx.x * TC_M;
-
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
-                     "r"(TC_N));
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-        asm volatile("tcgen05.fence::before_thread_sync;");
-    }
-    if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&mbar)), "r"(1));
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    // the rows' graph data (rows past N: element 0's corners; empty CSR rows)
-    if (KIND == 0) {
-        for (int r = tid; r < TC_M; r += TC_THREADS) {
-            const int4 v = n0 + r < N ? a.etri[n0 + r] : make_int4(0, 0, 0, 0);
-            s_tri[r] = v.x;
-            s_tri[TC_M + r] = v.y;
-            s_tri[2 * TC_M + r] = v.z;
-        }
-    } else {
-        for (int r = tid; r <= TC_M; r += TC_THREADS) s_off[r] = a.voff[min(n0 + r, N)];
-    }
-    // B tile: the packed image of W^T, copied as is
-#pragma unroll 4
-    for (int c = tid; c < TC_N * KC; c += TC_THREADS) Bs[c] = Wp[c];
-    __syncthreads();
-    const int qbase = KIND == 1 ? s_off[0] : 0;
-    const bool inc_smem = KIND == 1 && s_off[TC_M] - qbase <= MSG_INC_CAP;
-    if (KIND == 1 && inc_smem) {
-        for (int t = tid; t < s_off[TC_M] - qbase; t += TC_THREADS) {
-            const int e = a.vinc[qbase + t] >> 2;
-            s_inc[t] = e;
-            s_area[t] = a.earea[e];
-        }
-        __syncthreads();
-    }
-    // A tile: item it is row r = 8 rg + rl and the 8 hidden channels 8 cg .. 8 cg + 7; it forms
-    // the row's 16-byte chunk of each block of Z for those channels (chunk kc of row r sits at
-    // (rg KC + kc) 8 + rl). Consecutive threads take consecutive rows of one core matrix, so
-    // the shared-memory stores do not conflict.
-    constexpr int PER = TC_M * (TC_N / 8) / TC_THREADS;
-    static_assert(PER % 2 == 0, "items per thread must be even");
-#pragma unroll 1
-    for (int u = 0; u < PER; u += 2) {
-        int r[2], cg[2], n[2];
-#pragma unroll
-        for (int w = 0; w < 2; w++) {
-            const int it = tid + (u + w) * TC_THREADS;
-            r[w] = (it >> 6) * 8 + (it & 7);
-            cg[w] = (it >> 3) & 7;
-            n[w] = n0 + r[w];
-        }
-        float hs[2][8], m0[2][8], m1[2][8];
-        if (KIND == 0) {
-            float h0[2][8], h1[2][8], h2[2][8];
-            float4 g[2];
-#pragma unroll
-            for (int w = 0; w < 2; w++) {
-                const int c8 = cg[w] * 8, nc = min(n[w], N - 1);
-                g[w] = a.egrad[nc];
-                load8(a.hself + (size_t)nc * TC_N + c8, hs[w]);
-                load8(a.hother + (size_t)s_tri[r[w]] * TC_N + c8, h0[w]);
-                load8(a.hother + (size_t)s_tri[TC_M + r[w]] * TC_N + c8, h1[w]);
-                load8(a.hother + (size_t)s_tri[2 * TC_M + r[w]] * TC_N + c8, h2[w]);
-            }
-#pragma unroll
-            for (int w = 0; w < 2; w++) {
-#pragma unroll
-                for (int t = 0; t < 8; t++) {
-                    const float2 m = msg_elem_grad(g[w], h0[w][t], h1[w][t], h2[w][t], a.L);
-                    m0[w][t] = m.x;
-                    m1[w][t] = m.y;
-                }
-            }
-        } else {
-#pragma unroll
-            for (int w = 0; w < 2; w++) load8(a.hself + (size_t)min(n[w], N - 1) * TC_N + cg[w] * 8, hs[w]);
-#pragma unroll
-            for (int w = 0; w < 2; w++) {
-                const int c8 = cg[w] * 8;
-                const int q0 = s_off[r[w]], q1 = s_off[r[w] + 1];
-#pragma unroll
-                for (int t = 0; t < 8; t++) m0[w][t] = 0.0f;
-                // four incidences' rows in flight, summed in incidence order
-                int q = q0;
-                for (; q + 4 <= q1; q += 4) {
-                    float h[4][8], ar[4];
-#pragma unroll
-                    for (int j = 0; j < 4; j++) {
-                        const int e = inc_smem ? s_inc[q + j - qbase] : a.vinc[q + j] >> 2;
-                        ar[j] = inc_smem ? s_area[q + j - qbase] : a.earea[e];
-                        load8(a.hother + (size_t)e * TC_N + c8, h[j]);
-                    }
-#pragma unroll
-                    for (int j = 0; j < 4; j++)
-#pragma unroll
-                        for (int t = 0; t < 8; t++) m0[w][t] = msg_vert_acc(m0[w][t], ar[j], h[j][t]);
-                }
-                for (; q < q1; q++) {
-                    const int e = inc_smem ? s_inc[q - qbase] : a.vinc[q] >> 2;
-                    const float ar = inc_smem ? s_area[q - qbase] : a.earea[e];
-                    float h[8];
-                    load8(a.hother + (size_t)e * TC_N + c8, h);
-#pragma unroll
-                    for (int t = 0; t < 8; t++) m0[w][t] = msg_vert_acc(m0[w][t], ar, h[t]);
-                }
-                const float inv = a.vinvA[min(n[w], N - 1)];
-#pragma unroll
-                for (int t = 0; t < 8; t++) m0[w][t] = msg_vert_mean(m0[w][t], inv);
-            }
-        }
-#pragma unroll
-        for (int w = 0; w < 2; w++) {
-            if (n[w] >= N) {
-#pragma unroll
-                for (int t = 0; t < 8; t++) hs[w][t] = m0[w][t] = m1[w][t] = 0.0f;
-            }
-            uint4 *chunk = As + (size_t)(r[w] >> 3) * KC * 8 + (r[w] & 7);    // chunk kc at chunk[kc * 8]
-            chunk[cg[w] * 8] = pack_bf16x8(hs[w]);
-            chunk[(8 + cg[w]) * 8] = pack_bf16x8(m0[w]);
-            if (KIND == 0) chunk[(16 + cg[w]) * 8] = pack_bf16x8(m1[w]);
-        }
-    }
-    // make the generic-proxy writes of the tiles visible to the tensor core (async proxy)
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    __syncthreads();
-    const uint32_t tmem = tmem_base;
-    // the epilogue's residual rows, requested before the MMAs are issued: this thread's row and
-    // 32 columns (rows past N read row N - 1 and store nothing)
-    const int quarter = warp & 3, half = warp >> 2;
-    const int erow = n0 + quarter * 32 + lane;
-    float4 hres[8];
-    {
-        const float4 *hsrc = reinterpret_cast<const float4 *>(a.hself + (size_t)min(erow, N - 1) * TC_N + half * 32);
-#pragma unroll
-        for (int t = 0; t < 8; t++) hres[t] = hsrc[t];
-    }
-
-    if (tid == 0) {
-        asm volatile("tcgen05.fence::after_thread_sync;");
-        const uint32_t a0 = smem_u32(As), b0 = smem_u32(Bs);
-        constexpr uint32_t idesc = idesc_bf16_f32(TC_M, TC_N);
-#pragma unroll
-        for (int ks = 0; ks < K / 16; ks++) {
-            const uint64_t ad = umma_desc(a0 + ks * 256, 128, KC * 128);
-            const uint64_t bd = umma_desc(b0 + ks * 256, 128, KC * 128);
-            asm volatile(
-                "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-                "l"(ad), "l"(bd), "r"(idesc), "r"(ks));
-        }
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                         smem_u32(&mbar))
-                     : "memory");
-        bool ok = mbar_wait(smem_u32(&mbar), wait_cycles);
-        if (!ok) {
-            atomicOr(status, 2u);
-            // the MMAs may still be in flight: give them one more budget before TMEM is freed
-            mbar_wait(smem_u32(&mbar), wait_cycles);
-        }
-        s_ok = ok;
-    }
-    __syncthreads();
-
-    if (s_ok) {
-        asm volatile("tcgen05.fence::after_thread_sync;");
-        const int n = erow;
-        const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16);
-#pragma unroll
-        for (int q = 2 * half; q < 2 * half + 2; q++) {
-            float acc[16];
-            tmem_ld16(taddr + q * 16, acc);
-            if (n < N) {
-                float4 *dy = a.Y ? reinterpret_cast<float4 *>(a.Y + (size_t)n * TC_N + q * 16) : nullptr;
-                float4 *dh = reinterpret_cast<float4 *>(a.hnext + (size_t)n * TC_N + q * 16);
-#pragma unroll
-                for (int t = 0; t < 16; t += 4) {
-                    float y[4];
-#pragma unroll
-                    for (int u = 0; u < 4; u++) y[u] = tanhf(__fadd_rn(acc[t + u], bias[q * 16 + t + u]));
-                    const float4 h = hres[(q - 2 * half) * 4 + t / 4];
-                    if (dy) dy[t / 4] = make_float4(y[0], y[1], y[2], y[3]);
-                    dh[t / 4] = make_float4(__fadd_rn(h.x, y[0]), __fadd_rn(h.y, y[1]), __fadd_rn(h.z, y[2]),
-                                            __fadd_rn(h.w, y[3]));
-                }
-            }
-        }
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;");
-    __syncthreads();
-    if (warp == 0) {
-        asm volatile("tcgen05.fence::after_thread_sync;");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TC_N));
-    }
-}
-
-// ---------------------------------------------------------------------------------
-// The two backward contractions of a message layer (inputs Z [N][K] holding bfloat16 values,
-// K = 128 or 192; weights W [K][64]; dA = dL/d(pre-activation) [N][64], FP32):
-//   weight gradient  G[i][j] = sum_n Z[n][i] dA[n][j]           (k_wgrad_tc)
-//   input gradient   dZ[n][i] = sum_j dA[n][j] W[i][j]           (k_dgrad_tc)
-// dA is not a bfloat16 value, so each of its elements is split into two bfloat16 parts,
-// hi = bf16(dA) and lo = bf16(dA - hi), which carry 16 significant bits, and both parts
-// are multiplied: the products accumulate in FP32 in tensor memory. Operand tiles are
-// staged in the same K-major layout without swizzle as k_msg_layer_tc's (core matrices of 8
-// rows x 16 bytes, 128 bytes apart along K, KC * 128 bytes apart along M or N).
 
 __device__ __forceinline__ void split_bf16(float v, __nv_bfloat16 &hi, __nv_bfloat16 &lo)
 {
@@ -371,6 +138,120 @@ __device__ __forceinline__ void split_bf16(float v, __nv_bfloat16 &hi, __nv_bflo
 __device__ __forceinline__ uint32_t bf16x2_bits(__nv_bfloat16 a, __nv_bfloat16 b)
 {
     return (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
+}
+
+// Element incidences of a vertex-layer tile's rows held in shared memory (more go through
+// global memory, in the same order).
+constexpr int MSG_INC_CAP = 1536;
+
+// The turned accumulator: 128 rows of 64 floats, 68 apart (rows 17 x 16 bytes apart keep both
+// the row-wise stores and the octet-wise loads free of bank conflicts).
+constexpr int TURN_LD = 68;
+constexpr size_t TURN_BYTES = (size_t)TC_M * TURN_LD * 4;
+
+__host__ __device__ constexpr size_t cmax(size_t a, size_t b) { return a > b ? a : b; }
+
+// Graph data of a tile's rows: KIND 0 the three corners of 128 elements; KIND 1 the 129 CSR
+// offsets of the rows and the incidences (element << 2 | corner) and element areas of up to
+// MSG_INC_CAP incidences.
+__host__ __device__ constexpr size_t graph_smem(int kind)
+{
+    return kind == 0 ? (size_t)TC_M * 12 : (size_t)(TC_M + 4) * 4 + (size_t)MSG_INC_CAP * 8;
+}
+
+// Shared memory of k_msg_layer_tc: the A tile (128 x K bf16; the turned accumulator takes its
+// place), W^T (64 x K bf16), the graph data. Three CTAs fit an SM.
+__host__ __device__ constexpr size_t msg_a_smem(int kind)
+{
+    return cmax((size_t)TC_M * (kind == 0 ? 3 * TC_N : 2 * TC_N) * 2, TURN_BYTES);
+}
+__host__ __device__ constexpr size_t msg_layer_smem(int kind)
+{
+    return msg_a_smem(kind) + (size_t)TC_N * (kind == 0 ? 3 * TC_N : 2 * TC_N) * 2 + graph_smem(kind);
+}
+
+// The graph arrays of a layer and where a tile's share of them sits in shared memory.
+struct TileGraph {
+    int *tri;                    // KIND 0: [3][128]
+    int *off, *inc;              // KIND 1
+    float *area;
+    int qbase;
+    bool inc_smem;
+};
+
+template <int KIND>
+__device__ __forceinline__ TileGraph tile_graph_at(unsigned char *gdata)
+{
+    TileGraph g;
+    g.tri = reinterpret_cast<int *>(gdata);
+    g.off = reinterpret_cast<int *>(gdata);
+    g.inc = g.off + TC_M + 4;
+    g.area = reinterpret_cast<float *>(g.inc + MSG_INC_CAP);
+    g.qbase = 0;
+    g.inc_smem = false;
+    return g;
+}
+
+// Load the graph data of rows n0 .. n0 + 127 (rows past N: element 0's corners; empty CSR
+// rows) so that every gather has its address at hand. Ends with a block barrier.
+template <int KIND>
+__device__ __forceinline__ void load_tile_graph(const MsgLayerArgs &a, int n0, TileGraph &g)
+{
+    if constexpr (KIND == 0) {
+        for (int r = threadIdx.x; r < TC_M; r += TC_THREADS) {
+            const int4 v = n0 + r < a.N ? a.etri[n0 + r] : make_int4(0, 0, 0, 0);
+            g.tri[r] = v.x;
+            g.tri[TC_M + r] = v.y;
+            g.tri[2 * TC_M + r] = v.z;
+        }
+    } else {
+        for (int r = threadIdx.x; r <= TC_M; r += TC_THREADS) g.off[r] = a.voff[min(n0 + r, a.N)];
+        __syncthreads();
+        g.qbase = g.off[0];
+        const int nq = g.off[TC_M] - g.qbase;
+        g.inc_smem = nq <= MSG_INC_CAP;
+        if (g.inc_smem) {
+            for (int t = threadIdx.x; t < nq; t += TC_THREADS) {
+                const int ek = a.vinc[g.qbase + t];
+                g.inc[t] = ek;
+                g.area[t] = a.earea[ek >> 2];
+            }
+        }
+    }
+    __syncthreads();
+}
+
+// Thread item u of a tile: row r and the 8 hidden channels 8 cg .. 8 cg + 7; eight consecutive
+// threads cover one row, so that each global access of a quarter warp is 256 contiguous bytes
+// (with eight rows per quarter, every lane's access was an L1 pass of its own: 88 % of the
+// L1 pipe, 334 us for the 910k-row element layer).
+constexpr int ITEMS = TC_M * (TC_N / 8) / TC_THREADS;
+__device__ __forceinline__ int item_row(int u) { return ((int)threadIdx.x >> 3) + u * (TC_THREADS / 8); }
+__device__ __forceinline__ int item_cg() { return (int)threadIdx.x & 7; }
+
+// A staged tile of 128 rows: blocks of 64 features (128 rows x 128 bytes, swizzled), one after
+// another. Where chunk cg (8 features) of row r of block k sits, in 16-byte units.
+constexpr int TILE_BLOCK = TC_M * TC_N * 2;   // bytes
+__device__ __forceinline__ int tile_chunk(int r, int cg, int k)
+{
+    return k * (TILE_BLOCK / 16) + r * 8 + (cg ^ (r & 7));
+}
+
+// Read the accumulator's columns [col, col + 64) into the turned tile: warp w reads lanes
+// 32 (w % 4) .. + 31 and 32 columns. The caller synchronises the block before the tile is read.
+__device__ __forceinline__ void turn_tile(uint32_t tmem_col, float *turn)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, quarter = warp & 3, half = warp >> 2;
+    const uint32_t taddr = tmem_col + ((uint32_t)(quarter * 32) << 16);
+    float *row = turn + (size_t)(quarter * 32 + lane) * TURN_LD;
+#pragma unroll
+    for (int q = 2 * half; q < 2 * half + 2; q++) {
+        float v[16];
+        tmem_ld16(taddr + q * 16, v);
+#pragma unroll
+        for (int t = 0; t < 16; t += 4)
+            *reinterpret_cast<float4 *>(row + q * 16 + t) = make_float4(v[t], v[t + 1], v[t + 2], v[t + 3]);
+    }
 }
 
 __device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t ad, uint64_t bd, uint32_t idesc, int accumulate)
@@ -387,7 +268,7 @@ __device__ __forceinline__ void mma_commit(uint32_t bar)
 }
 
 // Bounded wait on phase `parity` of an mbarrier; false when the budget ran out.
-__device__ __forceinline__ bool mbar_wait_parity(uint32_t bar, uint32_t parity, long long budget)
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, long long budget)
 {
     const long long t0 = clock64();
     while (true) {
@@ -402,36 +283,45 @@ __device__ __forceinline__ bool mbar_wait_parity(uint32_t bar, uint32_t parity, 
     }
 }
 
-constexpr int WG_THREADS = 256;
-constexpr int WG_NC = 64;          // rows n of one staged chunk: 4 MMA steps of 16
-constexpr int WG_KC = WG_NC / 8;   // core matrices along the reduction in a chunk
-
-// Weight gradient: CTA b sums rows [b R, b R + R) of Z^T dA into partial[b][i * 64 + j], and
-// the bias gradient (the column sums of dA) into partial[b][K * 64 + j]. D is one (K = 128)
-// or two (K = 192: rows 128..191 and 64 rows of zeros) tiles of 128 x 64 in TMEM.
-template <int K>
-__global__ void __launch_bounds__(WG_THREADS)
-k_wgrad_tc(int N, int rows_per_cta, const float *__restrict__ Z, const float *__restrict__ dA,
-           float *__restrict__ partial, unsigned *__restrict__ status, long long wait_cycles)
+// The wait for committed MMAs: a wait that gives up flags the timeout and waits one more budget,
+// so that TMEM is not freed under MMAs still in flight.
+__device__ __forceinline__ bool mma_wait(uint32_t bar, uint32_t parity, long long budget, unsigned *status)
 {
-    constexpr int MT = (K + 127) / 128;
-    constexpr int A_CHUNKS = MT * 128 * WG_KC;     // 16-byte chunks of the A tile (rows i, K-major)
-    constexpr int B_CHUNKS = TC_N * WG_KC;         // of each B tile (rows j)
+    if (mbar_wait(bar, parity, budget)) return true;
+    atomicOr(status, 2u);
+    mbar_wait(bar, parity, budget);
+    return false;
+}
+
+// One message layer of the surrogate's forward pass (KIND 0: element rows, K = 192; KIND 1:
+// vertex rows, K = 128): the CTA forms 128 rows of Z from the hidden states while it
+// stages them as the A tile, so Z never goes to memory, then Y = tanh(Z W + b) and
+// h_next = h + Y. Bound by the gathers of the hidden states (1.5 KB of FP32 rows per element
+// row, 2 KB per vertex row, most of it from L2): persistent CTAs load W once, the rows' own
+// hidden states stay in registers for the residual, and results leave coalesced (before, each
+// lane stored its own row: 32 partial lines per store). Level 8 (459k vertices, 910k triangles):
+// element layer 462 -> 190 us, vertex layer 313 -> 133 us.
+template <int KIND>
+__global__ void __launch_bounds__(TC_THREADS, 3)
+k_msg_layer_tc(const MsgLayerArgs a, const uint4 *__restrict__ Wp, const float *__restrict__ bias,
+               unsigned *__restrict__ status, long long wait_cycles)
+{
+    constexpr int K = KIND == 0 ? 3 * TC_N : 2 * TC_N;
+    constexpr int KC = K / 8;    // core matrices along K
     extern __shared__ __align__(1024) unsigned char smem[];
-    uint4 *As = reinterpret_cast<uint4 *>(smem);
-    uint4 *Bh = As + A_CHUNKS;
-    uint4 *Bl = Bh + B_CHUNKS;
+    uint4 *As = reinterpret_cast<uint4 *>(smem);                              // 128 x K bf16
+    float *turn = reinterpret_cast<float *>(smem);                            // in its place after the MMAs
+    uint4 *Bs = reinterpret_cast<uint4 *>(smem + msg_a_smem(KIND));           // 64 x K bf16 (W^T)
+    TileGraph g = tile_graph_at<KIND>(smem + msg_a_smem(KIND) + (size_t)TC_N * K * 2);
     __shared__ __align__(8) uint64_t mbar;
     __shared__ uint32_t tmem_base;
     __shared__ int s_ok;
-    __shared__ float s_bias[WG_KC][TC_N];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int r0 = blockIdx.x * rows_per_cta, r1 = min(N, r0 + rows_per_cta);
-    const int nchunk = r1 > r0 ? (r1 - r0 + WG_NC - 1) / WG_NC : 0;
+    const int tid = threadIdx.x, warp = tid >> 5;
+    const int N = a.N, ntile = (N + TC_M - 1) / TC_M;
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
-                     "r"(MT * TC_N));
+                     "r"(TC_N));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
         asm volatile("tcgen05.fence::before_thread_sync;");
     }
@@ -440,126 +330,383 @@ k_wgrad_tc(int N, int rows_per_cta, const float *__restrict__ Z, const float *__
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         s_ok = 1;
     }
-    // rows K .. MT * 128 - 1 of A stay zero
-    for (int c = tid; c < A_CHUNKS; c += WG_THREADS) As[c] = make_uint4(0u, 0u, 0u, 0u);
-    // bias: thread t < 128 owns row octet t / 16 and columns 4 (t % 16) .. + 3 of every chunk
-    float bsum[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    __syncthreads();
-    const uint32_t tmem = tmem_base;
-    const uint32_t bar = smem_u32(&mbar);
-    const uint32_t a0 = smem_u32(As), bh0 = smem_u32(Bh), bl0 = smem_u32(Bl);
-    constexpr uint32_t idesc = idesc_bf16_f32(128, TC_N);
-
-    for (int ch = 0; ch < nchunk; ch++) {
-        const int n0 = r0 + ch * WG_NC;
-        // A: unit (octet oc, feature quad fq) reads Z[n0 + 8 oc + t][4 fq .. 4 fq + 3], t < 8,
-        // and writes the core-matrix rows of features 4 fq .. 4 fq + 3
-        for (int u = tid; u < WG_KC * (K / 4); u += WG_THREADS) {
-            const int oc = u / (K / 4), fq = u % (K / 4);
-            float4 v[8];
+    // B tile: the packed image of W^T, copied as is
+#pragma unroll 4
+    for (int c = tid; c < TC_N * KC; c += TC_THREADS) Bs[c] = Wp[c];
+    const int cg = item_cg(), c8 = cg * 8;
+    uint32_t parity = 0;
+    for (int tile = blockIdx.x; tile < ntile; tile += gridDim.x, parity ^= 1u) {
+        const int n0 = tile * TC_M;
+        load_tile_graph<KIND>(a, n0, g);
+        float hs[ITEMS][8];
 #pragma unroll
-            for (int t = 0; t < 8; t++) {
-                const int n = n0 + 8 * oc + t;
-                v[t] = n < r1 ? *reinterpret_cast<const float4 *>(Z + (size_t)n * K + 4 * fq)
-                              : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            }
-            const float *f = reinterpret_cast<const float *>(v);
+        for (int u = 0; u < ITEMS; u++) {
+            const int r = item_row(u), n = n0 + r, nc = min(n, N - 1);
+            float m0[8], m1[8];
+            if (KIND == 0) {
+                float h0[8], h1[8], h2[8];
+                const float4 gr = a.egrad[nc];
+                load8(a.hself + (size_t)nc * TC_N + c8, hs[u]);
+                load8(a.hother + (size_t)g.tri[r] * TC_N + c8, h0);
+                load8(a.hother + (size_t)g.tri[TC_M + r] * TC_N + c8, h1);
+                load8(a.hother + (size_t)g.tri[2 * TC_M + r] * TC_N + c8, h2);
 #pragma unroll
-            for (int q = 0; q < 4; q++) {
-                const int i = 4 * fq + q;
-                uint32_t w[4];
-#pragma unroll
-                for (int t = 0; t < 8; t += 2)
-                    w[t / 2] = bf16x2_bits(__float2bfloat16_rn(f[4 * t + q]), __float2bfloat16_rn(f[4 * (t + 1) + q]));
-                As[((i >> 3) * WG_KC + oc) * 8 + (i & 7)] = make_uint4(w[0], w[1], w[2], w[3]);
-            }
-        }
-        // B: the same for dA, split into hi and lo parts
-        if (tid < WG_KC * (TC_N / 4)) {
-            const int oc = tid / (TC_N / 4), jq = tid % (TC_N / 4);
-            float4 v[8];
-#pragma unroll
-            for (int t = 0; t < 8; t++) {
-                const int n = n0 + 8 * oc + t;
-                v[t] = n < r1 ? *reinterpret_cast<const float4 *>(dA + (size_t)n * TC_N + 4 * jq)
-                              : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            }
-            const float *f = reinterpret_cast<const float *>(v);
-#pragma unroll
-            for (int q = 0; q < 4; q++) {
-                const int j = 4 * jq + q;
-                uint32_t wh[4], wl[4];
-#pragma unroll
-                for (int t = 0; t < 8; t += 2) {
-                    __nv_bfloat16 h0, l0, h1, l1;
-                    split_bf16(f[4 * t + q], h0, l0);
-                    split_bf16(f[4 * (t + 1) + q], h1, l1);
-                    wh[t / 2] = bf16x2_bits(h0, h1);
-                    wl[t / 2] = bf16x2_bits(l0, l1);
+                for (int t = 0; t < 8; t++) {
+                    const float2 m = msg_elem_grad(gr, h0[t], h1[t], h2[t], a.L);
+                    m0[t] = m.x;
+                    m1[t] = m.y;
                 }
-                const int c = ((j >> 3) * WG_KC + oc) * 8 + (j & 7);
-                Bh[c] = make_uint4(wh[0], wh[1], wh[2], wh[3]);
-                Bl[c] = make_uint4(wl[0], wl[1], wl[2], wl[3]);
+            } else {
+                load8(a.hself + (size_t)nc * TC_N + c8, hs[u]);
+                const int q0 = g.off[r], q1 = g.off[r + 1];
 #pragma unroll
-                for (int t = 0; t < 8; t++) bsum[q] += f[4 * t + q];
+                for (int t = 0; t < 8; t++) m0[t] = 0.0f;
+                // three incidences' rows in flight, summed in incidence order
+                for (int q = q0; q < q1; q += 3) {
+                    float h[3][8], ar[3];
+#pragma unroll
+                    for (int j = 0; j < 3; j++) {
+                        const int qj = min(q + j, q1 - 1);
+                        const int e = (g.inc_smem ? g.inc[qj - g.qbase] : a.vinc[qj]) >> 2;
+                        ar[j] = g.inc_smem ? g.area[qj - g.qbase] : a.earea[e];
+                        load8(a.hother + (size_t)e * TC_N + c8, h[j]);
+                    }
+#pragma unroll
+                    for (int j = 0; j < 3; j++)
+                        if (q + j < q1)
+#pragma unroll
+                            for (int t = 0; t < 8; t++) m0[t] = msg_vert_acc(m0[t], ar[j], h[j][t]);
+                }
+                const float inv = a.vinvA[nc];
+#pragma unroll
+                for (int t = 0; t < 8; t++) m0[t] = msg_vert_mean(m0[t], inv);
             }
+            if (n >= N) {
+#pragma unroll
+                for (int t = 0; t < 8; t++) hs[u][t] = m0[t] = m1[t] = 0.0f;
+            }
+            As[tile_chunk(r, cg, 0)] = pack_bf16x8(hs[u]);
+            As[tile_chunk(r, cg, 1)] = pack_bf16x8(m0);
+            if (KIND == 0) As[tile_chunk(r, cg, 2)] = pack_bf16x8(m1);
         }
+        // make the generic-proxy writes of the tiles visible to the tensor core (async proxy)
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;");
         __syncthreads();
+        const uint32_t tmem = tmem_base;
         if (tid == 0) {
             asm volatile("tcgen05.fence::after_thread_sync;");
+            const uint32_t a0 = smem_u32(As), b0 = smem_u32(Bs);
+            constexpr uint32_t idesc = idesc_bf16_f32(TC_M, TC_N);
 #pragma unroll
-            for (int ks = 0; ks < WG_KC / 2; ks++) {
-                const uint64_t bdh = umma_desc(bh0 + ks * 256, 128, WG_KC * 128);
-                const uint64_t bdl = umma_desc(bl0 + ks * 256, 128, WG_KC * 128);
-#pragma unroll
-                for (int mt = 0; mt < MT; mt++) {
-                    const uint64_t ad = umma_desc(a0 + mt * 16 * WG_KC * 128 + ks * 256, 128, WG_KC * 128);
-                    mma_bf16(tmem + mt * TC_N, ad, bdh, idesc, ch > 0 || ks > 0);
-                    mma_bf16(tmem + mt * TC_N, ad, bdl, idesc, 1);
-                }
-            }
-            mma_commit(bar);
-            // the tiles are overwritten by the next chunk only after the products have read them
-            if (!mbar_wait_parity(bar, ch & 1, wait_cycles)) {
-                atomicOr(status, 2u);
-                mbar_wait_parity(bar, ch & 1, wait_cycles);
-                s_ok = 0;
-            }
+            for (int ks = 0; ks < K / 16; ks++)
+                mma_bf16(tmem, umma_desc_sw(a0 + (ks >> 2) * TILE_BLOCK + (ks & 3) * 32, 16, 1024),
+                         umma_desc(b0 + ks * 256, 128, KC * 128), idesc, ks);
+            mma_commit(smem_u32(&mbar));
+            if (!mma_wait(smem_u32(&mbar), parity, wait_cycles, status)) s_ok = 0;
         }
         __syncthreads();
         if (!s_ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        turn_tile(tmem, turn);
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < ITEMS; u++) {
+            const int r = item_row(u), n = n0 + r;
+            float acc[8];
+            load8_turned(turn + (size_t)r * TURN_LD + c8, cg, acc);
+            if (n < N) {
+                float y[8];
+#pragma unroll
+                for (int t = 0; t < 8; t++) {
+                    y[t] = tanhf(__fadd_rn(acc[t], bias[c8 + t]));
+                    hs[u][t] = __fadd_rn(hs[u][t], y[t]);
+                }
+                if (a.Y) store8(a.Y + (size_t)n * TC_N + c8, y);
+                store8(a.hnext + (size_t)n * TC_N + c8, hs[u]);
+            }
+        }
+        __syncthreads();     // the next tile overwrites the turned one
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    if (warp == 0) {
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TC_N));
+    }
+}
+
+// ---------------------------------------------------------------------------------
+// Backward of a message layer (inputs Z [N][K] holding bfloat16 values, K = 128 or 192; weights
+// W [K][64]; incoming gradient dh [N][64] of h_next), one kernel:
+//   dh    = dh_in + the gradient that the layers behind sent through their messages (gathered
+//           here from g0, g1, where they are per row of the other kind)
+//   dA    = dh (1 - Y^2)                                         (FP32)
+//   G     = Z^T dA, column sums of dA: weight and bias gradient  (partial per CTA)
+//   dZ    = dA W^T; dh_out = dh + dZ[:, 0:64]; m0, m1 = the other 64-wide blocks of dZ, the
+//           gradients of the layer's messages
+// dA is not a bfloat16 value, so each of its elements is split into two bfloat16 parts,
+// hi = bf16(dA) and lo = bf16(dA - hi), which carry 16 significant bits, and both parts
+// are multiplied: the products accumulate in FP32 in tensor memory.
+//
+// One staged tile serves both products: for dA W^T the rows are the M (K-major A operand), for
+// Z^T dA they are the reduction, which reads the same tile as MN-major operands. Before, Z, dA and dZ
+// went through memory in six kernels per layer: 7.1 GB per layer at level 8 (459k vertices, 910k
+// triangles), 2.2 ms; here 2.9 GB, 0.79 ms. Bound by the latency of the gathers.
+// TMEM: columns 0..127 dZ (the third block of a K = 192 layer takes columns 0..63 once they are
+// read), 128..191 G of features 0..127, 192..255 G of features 64..191 (its upper half is kept).
+template <int KIND, int INIT>
+__global__ void __launch_bounds__(TC_THREADS, 2)
+k_bwd_layer_tc(const BwdLayerArgs b, unsigned *__restrict__ status, long long wait_cycles)
+{
+    constexpr int K = KIND == 0 ? 3 * TC_N : 2 * TC_N;
+    constexpr int DC = TC_N / 8;                   // core matrices along the channels of W
+    constexpr int P = KIND == 0 ? 4 : 1;           // INIT: outputs behind the last layer
+    const MsgLayerArgs &a = b.m;
+    extern __shared__ __align__(1024) unsigned char smem[];
+    uint4 *Zs = reinterpret_cast<uint4 *>(smem);                              // 128 x K bf16
+    float *turn = reinterpret_cast<float *>(smem);                            // over Zs (and Ah) after the MMAs
+    uint4 *Ah = reinterpret_cast<uint4 *>(smem + (size_t)TC_M * K * 2);       // 128 x 64 bf16
+    uint4 *Al = Ah + TC_M * DC;
+    uint4 *Ws = Al + TC_M * DC;                                               // K x 64 bf16
+    TileGraph g = tile_graph_at<KIND>(reinterpret_cast<unsigned char *>(Ws + K * DC));
+    __shared__ __align__(8) uint64_t mbar[2];
+    __shared__ uint32_t tmem_base;
+    __shared__ int s_ok;
+    __shared__ float s_w[P][TC_N];
+    float *s_bias = turn;                                                     // [32][64], after the last tile
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int N = a.N, ntile = (N + TC_M - 1) / TC_M;
+
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
+                     "r"(256));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+        asm volatile("tcgen05.fence::before_thread_sync;");
+    }
+    if (tid == 0) {
+        for (int k = 0; k < 2; k++)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&mbar[k])), "r"(1));
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        s_ok = 1;
+    }
+    // W: chunk (row i = 8 ig + il, channels 8 kc .. + 7) is 16 contiguous bytes
+    for (int c = tid; c < K * DC; c += TC_THREADS) {
+        const int il = c & 7, kc = (c >> 3) % DC, ig = (c >> 3) / DC;
+        Ws[c] = reinterpret_cast<const uint4 *>(b.W)[(size_t)(ig * 8 + il) * DC + kc];
+    }
+    if (INIT)
+        for (int c = tid; c < P * TC_N; c += TC_THREADS)    // Wout is 64 x P
+            s_w[c % P][c / P] = __bfloat162float(b.Wout[c]);
+    const int cg = item_cg(), c8 = cg * 8;
+    float bsum[8];
+#pragma unroll
+    for (int t = 0; t < 8; t++) bsum[t] = 0.0f;
+    uint32_t parity = 0;
+    int done = 0;
+    for (int tile = blockIdx.x; tile < ntile; tile += gridDim.x, parity ^= 1u, done++) {
+        const int n0 = tile * TC_M;
+        load_tile_graph<KIND>(a, n0, g);
+        float dh[ITEMS][8];
+#pragma unroll
+        for (int u = 0; u < ITEMS; u++) {
+            const int r = item_row(u), n = n0 + r, nc = min(n, N - 1);
+            float hs[8], m0[8], m1[8], y[8];
+            load8(a.hself + (size_t)nc * TC_N + c8, hs);
+            load8(b.Y + (size_t)nc * TC_N + c8, y);
+            if (INIT) {
+#pragma unroll
+                for (int t = 0; t < 8; t++) {
+                    float s = 0.0f;
+#pragma unroll
+                    for (int j = 0; j < P; j++) s = fmaf(b.dout[(size_t)nc * P + j], s_w[j][c8 + t], s);
+                    dh[u][t] = s;
+                }
+            } else {
+                load8(b.dh_in + (size_t)nc * TC_N + c8, dh[u]);
+            }
+            if (KIND == 0) {
+                float h[3][8], d[3][8], w[3];
+                const float4 gr = a.egrad[nc];
+                const float ar = a.earea[nc];
+#pragma unroll
+                for (int k = 0; k < 3; k++) {
+                    const int v = g.tri[k * TC_M + r];
+                    load8(a.hother + (size_t)v * TC_N + c8, h[k]);
+                    load8(b.g0 + (size_t)v * TC_N + c8, d[k]);
+                    w[k] = a.vinvA[v];
+                }
+#pragma unroll
+                for (int t = 0; t < 8; t++) {
+                    const float2 m = msg_elem_grad(gr, h[0][t], h[1][t], h[2][t], a.L);
+                    m0[t] = m.x;
+                    m1[t] = m.y;
+                    dh[u][t] += ar * (w[0] * d[0][t] + w[1] * d[1][t] + w[2] * d[2][t]);
+                }
+            } else {
+                float ds[8];
+#pragma unroll
+                for (int t = 0; t < 8; t++) m0[t] = ds[t] = 0.0f;
+                const int q1 = g.off[r + 1];
+                for (int q = g.off[r]; q < q1; q++) {
+                    const int ek = g.inc_smem ? g.inc[q - g.qbase] : a.vinc[q], e = ek >> 2, k = ek & 3;
+                    const float ar = g.inc_smem ? g.area[q - g.qbase] : a.earea[e];
+                    float h[8];
+                    load8(a.hother + (size_t)e * TC_N + c8, h);
+                    if (!INIT) {
+                        float d0[8], d1[8];
+                        load8(b.g0 + (size_t)e * TC_N + c8, d0);
+                        load8(b.g1 + (size_t)e * TC_N + c8, d1);
+                        const float4 gr = a.egrad[e];
+                        const float gx = k == 0 ? gr.x : (k == 1 ? gr.z : -(gr.x + gr.z));
+                        const float gy = k == 0 ? gr.y : (k == 1 ? gr.w : -(gr.y + gr.w));
+#pragma unroll
+                        for (int t = 0; t < 8; t++) ds[t] += gx * d0[t] + gy * d1[t];
+                    }
+#pragma unroll
+                    for (int t = 0; t < 8; t++) m0[t] = msg_vert_acc(m0[t], ar, h[t]);
+                }
+                const float inv = a.vinvA[nc];
+#pragma unroll
+                for (int t = 0; t < 8; t++) {
+                    m0[t] = msg_vert_mean(m0[t], inv);
+                    if (!INIT) dh[u][t] += a.L * ds[t];
+                }
+            }
+            float dA[8];
+#pragma unroll
+            for (int t = 0; t < 8; t++) dA[t] = dh[u][t] * (1.0f - y[t] * y[t]);
+            if (n >= N) {
+#pragma unroll
+                for (int t = 0; t < 8; t++) hs[t] = m0[t] = m1[t] = dA[t] = 0.0f;
+            }
+            uint32_t wh[4], wl[4];
+#pragma unroll
+            for (int t = 0; t < 8; t += 2) {
+                __nv_bfloat16 x0, x1, l0, l1;
+                split_bf16(dA[t], x0, l0);
+                split_bf16(dA[t + 1], x1, l1);
+                wh[t / 2] = bf16x2_bits(x0, x1);
+                wl[t / 2] = bf16x2_bits(l0, l1);
+                bsum[t] += dA[t];
+                bsum[t + 1] += dA[t + 1];
+            }
+            Zs[tile_chunk(r, cg, 0)] = pack_bf16x8(hs);
+            Zs[tile_chunk(r, cg, 1)] = pack_bf16x8(m0);
+            if (KIND == 0) Zs[tile_chunk(r, cg, 2)] = pack_bf16x8(m1);
+            Ah[tile_chunk(r, cg, 0)] = make_uint4(wh[0], wh[1], wh[2], wh[3]);
+            Al[tile_chunk(r, cg, 0)] = make_uint4(wl[0], wl[1], wl[2], wl[3]);
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;");
+        __syncthreads();
+        const uint32_t tmem = tmem_base;
+        const uint32_t z0 = smem_u32(Zs), ah = smem_u32(Ah), al = smem_u32(Al), w0 = smem_u32(Ws);
+        if (tid == 0) {
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            // dZ[:, 0:128] = dA W[0:128]^T
+            constexpr uint32_t id1 = idesc_bf16_f32(TC_M, 128);
+#pragma unroll
+            for (int ks = 0; ks < DC / 2; ks++) {
+                const uint64_t bd = umma_desc(w0 + ks * 256, 128, DC * 128);
+                mma_bf16(tmem, umma_desc_sw(ah + ks * 32, 16, 1024), bd, id1, ks > 0);
+                mma_bf16(tmem, umma_desc_sw(al + ks * 32, 16, 1024), bd, id1, 1);
+            }
+            // G += Z^T dA: both operands MN-major (bits 15 and 16), 16 rows per step: the next 8 rows are
+            // the next 1024-byte group, the next 64 features the next block of the tile
+            constexpr uint32_t id2 = idesc_bf16_f32(TC_M, TC_N) | (1u << 15) | (1u << 16);
+#pragma unroll
+            for (int ks = 0; ks < TC_M / 16; ks++) {
+                const uint64_t bh = umma_desc_sw(ah + ks * 2048, TILE_BLOCK, 1024);
+                const uint64_t bl = umma_desc_sw(al + ks * 2048, TILE_BLOCK, 1024);
+#pragma unroll
+                for (int mt = 0; mt < (KIND == 0 ? 2 : 1); mt++) {
+                    const uint64_t ad = umma_desc_sw(z0 + mt * TILE_BLOCK + ks * 2048, TILE_BLOCK, 1024);
+                    mma_bf16(tmem + 128 + 64 * mt, ad, bh, id2, done > 0 || ks > 0);
+                    mma_bf16(tmem + 128 + 64 * mt, ad, bl, id2, 1);
+                }
+            }
+            mma_commit(smem_u32(&mbar[0]));
+            if (!mma_wait(smem_u32(&mbar[0]), parity, wait_cycles, status)) s_ok = 0;
+        }
+        __syncthreads();
+        if (!s_ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        turn_tile(tmem, turn);
+        asm volatile("tcgen05.fence::before_thread_sync;");
+        __syncthreads();
+        if (KIND == 0 && tid == 0) {
+            // dZ[:, 128:192] into the columns that were just read (Zs and the turned tile are not touched)
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            constexpr uint32_t id3 = idesc_bf16_f32(TC_M, TC_N);
+#pragma unroll
+            for (int ks = 0; ks < DC / 2; ks++) {
+                const uint64_t bd = umma_desc(w0 + 16 * DC * 128 + ks * 256, 128, DC * 128);
+                mma_bf16(tmem, umma_desc_sw(ah + ks * 32, 16, 1024), bd, id3, ks > 0);
+                mma_bf16(tmem, umma_desc_sw(al + ks * 32, 16, 1024), bd, id3, 1);
+            }
+            mma_commit(smem_u32(&mbar[1]));
+        }
+        auto put = [&](float *out, bool add) {
+#pragma unroll
+            for (int u = 0; u < ITEMS; u++) {
+                const int r = item_row(u), n = n0 + r;
+                float v[8];
+                load8_turned(turn + (size_t)r * TURN_LD + c8, cg, v);
+                if (add)
+#pragma unroll
+                    for (int t = 0; t < 8; t++) v[t] += dh[u][t];
+                if (n < N) store8(out + (size_t)n * TC_N + c8, v);
+            }
+            __syncthreads();
+        };
+        put(b.dh_out, true);
+        turn_tile(tmem + 64, turn);
+        __syncthreads();
+        put(b.m0, false);
+        if (KIND == 0) {
+            if (tid == 0 && !mma_wait(smem_u32(&mbar[1]), parity, wait_cycles, status)) s_ok = 0;
+            __syncthreads();
+            if (!s_ok) break;
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            turn_tile(tmem, turn);
+            __syncthreads();
+            put(b.m1, false);
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;");
     }
 
-    // bias partial: the 8 row octets' sums in a fixed order
-    if (tid < WG_KC * (TC_N / 4)) {
-        const int oc = tid / (TC_N / 4), jq = tid % (TC_N / 4);
+    // bias partial: the 32 threads of a channel octet, in a fixed order
+    __syncthreads();
+    {
+        const int part = tid >> 3;
 #pragma unroll
-        for (int q = 0; q < 4; q++) s_bias[oc][4 * jq + q] = bsum[q];
+        for (int t = 0; t < 8; t++) s_bias[part * TC_N + c8 + t] = bsum[t];
     }
     __syncthreads();
-    float *out = partial + (size_t)blockIdx.x * ((size_t)K * TC_N + TC_N);
+    float *out = b.partial + (size_t)blockIdx.x * ((size_t)K * TC_N + TC_N);
     if (tid < TC_N) {
-        float b = 0.0f;
-        for (int oc = 0; oc < WG_KC; oc++) b += s_bias[oc][tid];
-        out[(size_t)K * TC_N + tid] = b;
+        float x = 0.0f;
+        for (int k = 0; k < 32; k++) x += s_bias[k * TC_N + tid];
+        out[(size_t)K * TC_N + tid] = x;
     }
-    // G rows i = 128 mt + 32 (warp % 4) + lane, columns 32 (warp / 4) .. + 31
+    // G rows i: features 0..127 from the first accumulator, 128..191 from the second's lanes 64..127
     asm volatile("tcgen05.fence::after_thread_sync;");
+    const uint32_t tmem = tmem_base;
     const int quarter = warp & 3, half = warp >> 2;
 #pragma unroll
-    for (int mt = 0; mt < MT; mt++) {
-        const int i = mt * 128 + quarter * 32 + lane;
+    for (int mt = 0; mt < (KIND == 0 ? 2 : 1); mt++) {
+        const int i = mt * 64 + quarter * 32 + lane;
 #pragma unroll
         for (int q = 2 * half; q < 2 * half + 2; q++) {
             float v[16];
-            if (nchunk > 0 && s_ok) {
-                tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + mt * TC_N + q * 16, v);
+            if (s_ok) {
+                tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + 128 + 64 * mt + q * 16, v);
             } else {
 #pragma unroll
                 for (int t = 0; t < 16; t++) v[t] = 0.0f;
             }
-            if (i < K) {
+            if (mt == 0 || quarter >= 2) {
                 float4 *dst = reinterpret_cast<float4 *>(out + (size_t)i * TC_N + q * 16);
 #pragma unroll
                 for (int t = 0; t < 16; t += 4) dst[t / 4] = make_float4(v[t], v[t + 1], v[t + 2], v[t + 3]);
@@ -570,161 +717,34 @@ k_wgrad_tc(int N, int rows_per_cta, const float *__restrict__ Z, const float *__
     __syncthreads();
     if (warp == 0) {
         asm volatile("tcgen05.fence::after_thread_sync;");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(MT * TC_N));
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(256));
     }
 }
 
-// Input gradient: dZ[n][i] = sum_j dA[n][j] W[i][j] for 128 rows n per CTA; the reduction is
-// over the 64 output channels j (4 MMA steps, each on the hi and the lo part of dA), the MMA's
-// N is the layer's K (128 or 192 TMEM columns). W (K x 64 bfloat16, row-major) is already the
-// K-major image of the B operand: row i holds W[i][0 .. 63].
-template <int K>
-__global__ void __launch_bounds__(WG_THREADS)
-k_dgrad_tc(int N, const float *__restrict__ dA, const __nv_bfloat16 *__restrict__ W, float *__restrict__ dZ,
-           unsigned *__restrict__ status, long long wait_cycles)
+__host__ __device__ constexpr size_t bwd_layer_smem(int kind)
 {
-    constexpr int KC = TC_N / 8;                   // core matrices along the reduction (8)
-    constexpr int TCOLS = K <= 128 ? 128 : 256;    // TMEM allocation (a power of two)
-    extern __shared__ __align__(1024) unsigned char smem[];
-    uint4 *Ah = reinterpret_cast<uint4 *>(smem);   // 128 x 64 bf16
-    uint4 *Al = Ah + TC_M * KC;
-    uint4 *Bs = Al + TC_M * KC;                    // K x 64 bf16
-    __shared__ __align__(8) uint64_t mbar;
-    __shared__ uint32_t tmem_base;
-    __shared__ int s_ok;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int n0 = blockIdx.x * TC_M;
-
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
-                     "r"(TCOLS));
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-        asm volatile("tcgen05.fence::before_thread_sync;");
-    }
-    if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&mbar)), "r"(1));
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    // A: chunk (row r = 8 rg + rl, channels 8 kc .. + 7) of dA, split into hi and lo
-    for (int c = tid; c < TC_M * KC; c += WG_THREADS) {
-        const int rl = c & 7, kc = (c >> 3) % KC, rg = (c >> 3) / KC;
-        const int n = n0 + rg * 8 + rl;
-        float4 va = make_float4(0.0f, 0.0f, 0.0f, 0.0f), vb = va;
-        if (n < N) {
-            va = *reinterpret_cast<const float4 *>(dA + (size_t)n * TC_N + kc * 8);
-            vb = *reinterpret_cast<const float4 *>(dA + (size_t)n * TC_N + kc * 8 + 4);
-        }
-        const float f[8] = {va.x, va.y, va.z, va.w, vb.x, vb.y, vb.z, vb.w};
-        uint32_t wh[4], wl[4];
-#pragma unroll
-        for (int t = 0; t < 8; t += 2) {
-            __nv_bfloat16 h0, l0, h1, l1;
-            split_bf16(f[t], h0, l0);
-            split_bf16(f[t + 1], h1, l1);
-            wh[t / 2] = bf16x2_bits(h0, h1);
-            wl[t / 2] = bf16x2_bits(l0, l1);
-        }
-        Ah[(rg * KC + kc) * 8 + rl] = make_uint4(wh[0], wh[1], wh[2], wh[3]);
-        Al[(rg * KC + kc) * 8 + rl] = make_uint4(wl[0], wl[1], wl[2], wl[3]);
-    }
-    // B: chunk (row i = 8 ig + il, channels 8 kc .. + 7) is 16 contiguous bytes of W
-    const uint4 *Wv = reinterpret_cast<const uint4 *>(W);
-    for (int c = tid; c < K * KC; c += WG_THREADS) {
-        const int il = c & 7, kc = (c >> 3) % KC, ig = (c >> 3) / KC;
-        Bs[c] = Wv[(size_t)(ig * 8 + il) * KC + kc];
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    __syncthreads();
-    const uint32_t tmem = tmem_base;
-    if (tid == 0) {
-        asm volatile("tcgen05.fence::after_thread_sync;");
-        const uint32_t ah = smem_u32(Ah), al = smem_u32(Al), b0 = smem_u32(Bs);
-        constexpr uint32_t idesc = idesc_bf16_f32(TC_M, K);
-#pragma unroll
-        for (int ks = 0; ks < KC / 2; ks++) {
-            const uint64_t bd = umma_desc(b0 + ks * 256, 128, KC * 128);
-            mma_bf16(tmem, umma_desc(ah + ks * 256, 128, KC * 128), bd, idesc, ks > 0);
-            mma_bf16(tmem, umma_desc(al + ks * 256, 128, KC * 128), bd, idesc, 1);
-        }
-        mma_commit(smem_u32(&mbar));
-        bool ok = mbar_wait_parity(smem_u32(&mbar), 0, wait_cycles);
-        if (!ok) {
-            atomicOr(status, 2u);
-            mbar_wait_parity(smem_u32(&mbar), 0, wait_cycles);
-        }
-        s_ok = ok;
-    }
-    __syncthreads();
-    if (s_ok) {
-        asm volatile("tcgen05.fence::after_thread_sync;");
-        const int quarter = warp & 3, half = warp >> 2;
-        const int n = n0 + quarter * 32 + lane;
-        const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16);
-        constexpr int GROUPS = K / 16;             // 16-column groups, split between the two halves
-        for (int q = half; q < GROUPS; q += 2) {
-            float v[16];
-            tmem_ld16(taddr + q * 16, v);
-            if (n < N) {
-                float4 *dst = reinterpret_cast<float4 *>(dZ + (size_t)n * K + q * 16);
-#pragma unroll
-                for (int t = 0; t < 16; t += 4) dst[t / 4] = make_float4(v[t], v[t + 1], v[t + 2], v[t + 3]);
-            }
-        }
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;");
-    __syncthreads();
-    if (warp == 0) {
-        asm volatile("tcgen05.fence::after_thread_sync;");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TCOLS));
-    }
+    const size_t K = kind == 0 ? 3 * TC_N : 2 * TC_N;
+    return (size_t)TC_M * K * 2 + 2 * (size_t)TC_M * TC_N * 2 + K * TC_N * 2 + graph_smem(kind);
 }
 
 }  // namespace
 
 bool linear_tc_supported(int K, int P) { return P == TC_N && (K == 128 || K == 192); }
 
-size_t wgrad_tc_smem(int K) { return (size_t)((K + 127) / 128) * 128 * WG_NC * 2 + 2 * (size_t)TC_N * WG_NC * 2; }
+int bwd_layer_ctas(int N) { return std::max(1, std::min((N + TC_M - 1) / TC_M, 2 * 152)); }
 
-cudaError_t launch_wgrad_tc(int N, int K, int rows_per_cta, const float *Z, const float *dA, float *partial,
-                            unsigned *status, cudaStream_t st)
+cudaError_t launch_bwd_layer_tc(const BwdLayerArgs &b, unsigned *status, cudaStream_t st)
 {
-    if (rows_per_cta <= 0 || rows_per_cta % WG_NC) return cudaErrorInvalidValue;
-    const int grid = std::max(1, (N + rows_per_cta - 1) / rows_per_cta);
-    const size_t smem = wgrad_tc_smem(K);
-    cudaError_t e;
-    if (K == 128) {
-        if ((e = cudaFuncSetAttribute(k_wgrad_tc<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-            return e;
-        k_wgrad_tc<128><<<grid, WG_THREADS, smem, st>>>(N, rows_per_cta, Z, dA, partial, status, 2000000000ll);
-    } else if (K == 192) {
-        if ((e = cudaFuncSetAttribute(k_wgrad_tc<192>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-            return e;
-        k_wgrad_tc<192><<<grid, WG_THREADS, smem, st>>>(N, rows_per_cta, Z, dA, partial, status, 2000000000ll);
-    } else {
-        return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
-}
-
-cudaError_t launch_dgrad_tc(int N, int K, const float *dA, const __nv_bfloat16 *W, float *dZ, unsigned *status,
-                            cudaStream_t st)
-{
-    const int grid = (N + TC_M - 1) / TC_M;
-    if (grid == 0) return cudaSuccess;
-    const size_t smem = 2 * (size_t)TC_M * TC_N * 2 + (size_t)K * TC_N * 2;
-    cudaError_t e;
-    if (K == 128) {
-        if ((e = cudaFuncSetAttribute(k_dgrad_tc<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-            return e;
-        k_dgrad_tc<128><<<grid, WG_THREADS, smem, st>>>(N, dA, W, dZ, status, 2000000000ll);
-    } else if (K == 192) {
-        if ((e = cudaFuncSetAttribute(k_dgrad_tc<192>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-            return e;
-        k_dgrad_tc<192><<<grid, WG_THREADS, smem, st>>>(N, dA, W, dZ, status, 2000000000ll);
-    } else {
-        return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
+    const int grid = bwd_layer_ctas(b.m.N);
+    const size_t smem = bwd_layer_smem(b.m.kind);
+    const bool init = b.dout != nullptr;
+    const void *fn = b.m.kind == 0 ? (init ? (const void *)k_bwd_layer_tc<0, 1> : (const void *)k_bwd_layer_tc<0, 0>)
+                                   : (init ? (const void *)k_bwd_layer_tc<1, 1> : (const void *)k_bwd_layer_tc<1, 0>);
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    long long cycles = 2000000000ll;   // about one second
+    void *args[] = {const_cast<BwdLayerArgs *>(&b), &status, &cycles};
+    return cudaLaunchKernel(fn, dim3(grid), dim3(TC_THREADS), args, smem, st);
 }
 
 size_t linear_tc_packed_elems(int K) { return (size_t)TC_N * K; }
@@ -741,7 +761,7 @@ cudaError_t launch_msg_layer_tc(const MsgLayerArgs &a, const __nv_bfloat16 *pack
 {
     const uint4 *Wp = reinterpret_cast<const uint4 *>(packed);
     if (a.kind != 0 && a.kind != 1) return cudaErrorInvalidValue;
-    const int grid = (a.N + TC_M - 1) / TC_M;
+    const int grid = std::min((a.N + TC_M - 1) / TC_M, 3 * 152);   // three CTAs per SM
     if (grid == 0) return cudaSuccess;
     const size_t smem = msg_layer_smem(a.kind);
     const void *fn = a.kind == 0 ? (const void *)k_msg_layer_tc<0> : (const void *)k_msg_layer_tc<1>;
