@@ -117,7 +117,8 @@ typedef struct sesw_mesh {
  *                   before the start of a subcycle are taken equal to level 0 and <<U>> is the
  *                   mean of the AB3 transports, which keeps Eq. 4.11 exact. In
  *                   SESW_MODE_PERSISTENT, patches of at most 1536 slots and 768 own vertices
- *                   keep its state on chip and larger ones stream it from L2; patches too
+ *                   keep all their data on chip, larger ones stream the static slot data (and
+ *                   beyond 7 slots per thread also their state) from L2; patches too
  *                   large for the streaming kernel's shared memory give SESW_EINVAL (upload
  *                   in SESW_MODE_GRAPH instead)
  *   flags        bit 0 (SESW_FLAG_NO_STABILITY_CHECK): accept parameters whose Courant
@@ -201,8 +202,8 @@ typedef struct sesw_info {
     int32_t npack;           /* persistent mode: cooperative launches per step (packs of meshes
                                 that together fit the resident grid) */
     int32_t streamed;        /* persistent mode: nonzero when the (first) pack streams its transport,
-                                sums and static slot data from L2, for patches too large for
-                                registers: 1 with the slots' corner indices held in shared memory,
+                                sums and static slot data from L2 (SESM up to 7 slots per thread: only
+                                the static slot data), for patches too large for registers: 1 with the slots' corner indices held in shared memory,
                                 2 with them read from L2 too (the largest patches) */
     double visc_number;      /* viscous number of the barotropic viscosity (see sesw_params;
                                 0 until parameters are set) */

@@ -126,7 +126,7 @@ int capture_step_graph(sesw_ctx *c, int parity, cudaGraphExec_t *out)
     if (e != cudaSuccess) {
     } else if (c->mode == SESW_MODE_PERSISTENT) {
         e = c->params.scheme == 1
-                ? sesw::launch_persistent_sesm(c->dm, c->ds, c->args, c->params.M, parity, c->packs, c->cap_stream)
+                ? sesw::launch_persistent_sesm(c->dm, c->ds, c->args, c->params.M, parity, 1, c->packs, c->cap_stream)
                 : sesw::launch_persistent(c->dm, c->ds, c->args, c->params.M, parity, 1, c->groups, c->cap_stream);
     } else if (c->params.scheme == 1) {
         // SESM: level rings, U^m in B[m % 3] (B[0] holds U^0 and, at the end, U^M) and
@@ -203,7 +203,7 @@ int enqueue_step(sesw_ctx *c)
 {
     if (c->mode == SESW_MODE_PERSISTENT && !c->persist_graph_ok) {
         if (c->params.scheme == 1)
-            CK(c, sesw::launch_persistent_sesm(c->dm, c->ds, c->args, c->params.M, c->parity, c->packs, c->stream));
+            CK(c, sesw::launch_persistent_sesm(c->dm, c->ds, c->args, c->params.M, c->parity, 1, c->packs, c->stream));
         else
             CK(c, sesw::launch_persistent(c->dm, c->ds, c->args, c->params.M, c->parity, 1, c->groups, c->stream));
         c->parity ^= 1;
@@ -235,9 +235,14 @@ int enqueue_step(sesw_ctx *c)
 // failure test's silent patch.
 int steps_per_launch(const sesw_ctx *c, int n)
 {
-    if (c->mode != SESW_MODE_PERSISTENT || c->params.scheme != 0 || c->args.silent_patch >= 0) return 1;
-    for (const auto &g : c->groups)
-        if (g.plan.stream) return 1;
+    if (c->mode != SESW_MODE_PERSISTENT || c->args.silent_patch >= 0) return 1;
+    if (c->params.scheme == 1) {
+        for (const auto &pk : c->packs)
+            if (pk.plan_sesm.stream && !pk.plan_sesm.teams) return 1;
+    } else {
+        for (const auto &g : c->groups)
+            if (g.plan.stream) return 1;
+    }
     return std::min(n, std::max(1, 512 / c->params.M));
 }
 
@@ -531,9 +536,13 @@ static void make_packs(const sesw::HostMesh &hm, const std::vector<char> &large,
             }
             pk.plan.blocks_per_sm = kbps;
             if (streamed) {
-                pk.plan_sesm = sesw::persistent_plan_sesm_stream(pk.mx, kbps, idx_mode);
+                if (idx_mode != 0) pk.plan_sesm = sesw::persistent_plan_sesm_teams(pk.mx, kbps);
+                if (pk.plan_sesm.slots_per_thread == 0)
+                    pk.plan_sesm = sesw::persistent_plan_sesm_stream(pk.mx, kbps, idx_mode);
             } else {
                 pk.plan_sesm = sesw::persistent_plan_sesm(pk.mx, kbps);
+                if (kform == SESW_FORM_AUTO && pk.plan_sesm.slots_per_thread == 0)
+                    pk.plan_sesm = sesw::persistent_plan_sesm_teams(pk.mx, kbps);
                 if (kform == SESW_FORM_AUTO && pk.plan_sesm.slots_per_thread == 0)
                     pk.plan_sesm = sesw::persistent_plan_sesm_stream(pk.mx, kbps);
             }
@@ -808,8 +817,8 @@ static int upload_batch(sesw_ctx *c, const sesw_mesh *meshes, int n)
         for (const auto &pk : packs) {
             CK(c, pk.plan.stream ? sesw::persistent_prepare_stream(pk.plan) : sesw::persistent_prepare(pk.plan));
             if (plan_sesm.slots_per_thread > 0)
-                CK(c, pk.plan_sesm.stream ? sesw::persistent_prepare_sesm_stream(pk.plan_sesm)
-                                          : sesw::persistent_prepare_sesm(pk.plan_sesm));
+                CK(c, pk.plan_sesm.stream && !pk.plan_sesm.teams ? sesw::persistent_prepare_sesm_stream(pk.plan_sesm)
+                                                                 : sesw::persistent_prepare_sesm(pk.plan_sesm));
         }
     } else {
         TRY(zalloc(c, &s.eta_x[0], hm.nv, "eta_x"));
@@ -992,7 +1001,7 @@ static int set_params_impl(sesw_ctx *c, int n, const sesw_params *ps)
     // the streaming SESM kernel keeps U^{m-2} and U_AB^{m-1} in two more slot arrays
     if (p->scheme == 1 && c->mode == SESW_MODE_PERSISTENT && !c->ds.U_x[0]) {
         bool streamed = false;
-        for (const auto &pk : c->packs) streamed = streamed || pk.plan_sesm.stream;
+        for (const auto &pk : c->packs) streamed = streamed || (pk.plan_sesm.stream && !pk.plan_sesm.teams);
         if (streamed) {
             TRY(zalloc(c, &c->ds.U_x[0], (size_t)c->dm.nslot, "U_x"));
             TRY(zalloc(c, &c->ds.U_x[1], (size_t)c->dm.nslot, "U_x"));
@@ -1232,7 +1241,10 @@ int sesw_advance(sesw_ctx *c, int32_t nsteps)
     for (int n = 0; n < nsteps;) {
         const int k = steps_per_launch(c, nsteps - n);
         if (k > 1) {
-            CK(c, sesw::launch_persistent(c->dm, c->ds, c->args, c->params.M, c->parity, k, c->groups, c->stream));
+            if (c->params.scheme == 1)
+                CK(c, sesw::launch_persistent_sesm(c->dm, c->ds, c->args, c->params.M, c->parity, k, c->packs, c->stream));
+            else
+                CK(c, sesw::launch_persistent(c->dm, c->ds, c->args, c->params.M, c->parity, k, c->groups, c->stream));
             c->parity ^= 1;
         } else {
             TRY(enqueue_step(c));

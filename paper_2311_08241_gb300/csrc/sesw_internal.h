@@ -247,9 +247,10 @@ struct PersistentPlan {
     int cached = 0;             // 1: the patch's static data lives on chip (vertices' data in shared memory,
                                 // slots' in tensor memory; the SESM kernel: all in shared memory); 2: the same
                                 // except some of the slots' forcing and corner indices, read from L2
-    // the register SE kernel: a block per SM of `teams` teams, each with `threads` threads and its
-    // part of the shared memory; at most `grid` blocks, with tmem_cols tensor-memory columns each
-    int teams = 1, team_smem = 0, tmem_cols = 0, grid = 0;
+    // the kernels that run teams: a block per SM of `teams` teams, each with `threads` threads and its
+    // part of the shared memory; at most `grid` blocks, with tmem_cols tensor-memory columns each.
+    // teams = 0: a block per patch (the streaming kernels)
+    int teams = 0, team_smem = 0, tmem_cols = 0, grid = 0;
     int stream = 0;             // state and static data in global memory (the streaming kernels):
                                 // 1 with the corner indices in shared memory, 2 without
     int blocks_per_sm = 1;
@@ -294,13 +295,17 @@ PersistentPlan persistent_plan_stream(const PatchMax &mx, int blocks_per_sm, int
 cudaError_t persistent_prepare_stream(const PersistentPlan &plan);
 cudaError_t launch_persistent_stream_group(const DevMesh &m, const DevState &s, const StepArgs &a, int M, int parity,
                                            const PackGroup &g, cudaStream_t stream);
-// The SESM scheme in the persistent form (k_persistent_sesm): cached patches of at most
-// 4 x 384 slots and 2 x 384 own vertices; an empty plan when the patches do not fit.
+// The SESM scheme in the persistent form: cached patches of at most 4 x 384 slots and 2 x 384 own
+// vertices (k_persistent_sesm), or patches of up to 7 slots per thread whose state stays on
+// chip and whose static data stream from L2 (k_persistent_sesm_teams); an empty plan when the
+// patches do not fit.
 PersistentPlan persistent_plan_sesm(const PatchMax &mx, int blocks_per_sm);
+PersistentPlan persistent_plan_sesm_teams(const PatchMax &mx, int blocks_per_sm);
 cudaError_t persistent_prepare_sesm(const PersistentPlan &plan);
 // Fill m.slot_k from the slots' static data, g and each patch's substep length.
 cudaError_t launch_slot_coef(const DevMesh &m, float g, cudaStream_t stream);
-cudaError_t launch_persistent_sesm(const DevMesh &m, const DevState &s, const StepArgs &a, int M, int parity,
+// One launch per pack advances nsteps steps (1 where a pack runs k_persistent_sesm_stream).
+cudaError_t launch_persistent_sesm(const DevMesh &m, const DevState &s, const StepArgs &a, int M, int parity, int nsteps,
                                    const std::vector<PackPlan> &packs, cudaStream_t stream);
 
 struct Surrogate;

@@ -35,15 +35,6 @@ namespace {
 // elevation is exchanged like any other, and only the sums restart. A launch of n steps loads
 // the patch once instead of n times.
 
-constexpr int kMaxTeams = 4;
-
-
-// Barrier `bar` (1 ..) of a team of T threads (whole warps); barrier 0 is the block's.
-__device__ __forceinline__ void team_sync(int bar, int T)
-{
-    asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(T) : "memory");
-}
-
 __device__ __forceinline__ float4 slot_coef(const float4 c, float g, float dt)
 {
     const float aa = __fmul_rn(c.z, __fmul_rn(0.5f, dt));
@@ -108,11 +99,6 @@ __device__ __forceinline__ void persistent_patch(const PArgs &P, const int p, co
     // no per-thread condition. The fluxes of corners that are not own vertices, and of such empty
     // slots, go to one of 32 dummy words (one per lane).
     const uint32_t dummy = team + (uint32_t)P.off_dummy + 4u * (tid & 31);
-    auto flux_place = [&](uint32_t e) {
-        return e == 0x1fffffu ? dummy
-                              : team + (uint32_t)P.off_flux +
-                                    16u * (((e & 15u) >> 2) * (uint32_t)P.row_vertices + (e >> 4)) + 4u * (e & 3u);
-    };
     float2 u[SPT], shi[SPT], slo[kSloShared ? 1 : SPT];
 #pragma unroll
     for (int j = 0; j < SPT; j++) {
@@ -129,9 +115,9 @@ __device__ __forceinline__ void persistent_patch(const PArgs &P, const int p, co
             q.a1 = team + 4u * l.y;
             q.a2 = team + 4u * l.z;
             const uint2 f = in ? P.sf[s] : make_uint2(0xffffffffu, 0x7fffffffu);
-            q.f0 = flux_place(f.x & 0x1fffffu);
-            q.f1 = flux_place((f.x >> 21) | ((f.y & 0x3ffu) << 11));
-            q.f2 = flux_place((f.y >> 10) & 0x1fffffu);
+            q.f0 = flux_place(P, team, dummy, f.x & 0x1fffffu);
+            q.f1 = flux_place(P, team, dummy, (f.x >> 21) | ((f.y & 0x3ffu) << 11));
+            q.f2 = flux_place(P, team, dummy, (f.y >> 10) & 0x1fffffu);
             TS::store(tm, j, q);
             if (TS::kFluxShared && i < nsp) {
                 *reinterpret_cast<uint32_t *>(smem_raw + P.off_f01 + 4 * i) = (q.f0 >> 2) | (q.f1 << 14);
@@ -348,46 +334,6 @@ void *persistent_kernel(int spt, int nonlin, int cached, int extra)
 
 int tmem_words(int spt) { return spt <= 4 ? 16 * spt : (spt <= 6 ? 60 : 64); }
 
-// Shared memory of one team, from its largest patch: elevation of own and halo vertices; the
-// fluxes, then 32 dummy words; 1/A_v and halo ids; from 5 slots per thread the flux places, from
-// 6 the low parts of the compensated sums. Vertex-major fluxes (cached): each own vertex has a row
-// of one word per incidence (4 words per quad, quad k of all vertices in array k), which the
-// element pass fills and the vertex pass reads 16 bytes at a time, in the place of an
-// index row and eight dependent 4-byte reads (the reads' bank conflicts kept the
-// shared-memory pipe busy longer than the element pass). Not cached: three words per slot.
-struct SeLayout {
-    size_t flux, dummy, inv, halo, f01, f2, slo, total;
-    int quads;
-};
-
-SeLayout se_layout(const PatchMax &m, int spt, int cached)
-{
-    SeLayout L{};
-    const size_t slots = ((size_t)m.slots + 31) & ~(size_t)31;   // whole warps
-    size_t o = align16(sizeof(float) * (size_t)m.local);
-    L.flux = o;
-    if (!cached) {
-        L.total = align16(o + 12 * slots);
-        return L;
-    }
-    L.quads = std::max(2, (m.deg + 3) / 4);
-    o += 16 * (size_t)L.quads * (size_t)m.vertices;
-    L.dummy = o;
-    o += 128;
-    L.inv = o;
-    o = align16(o + sizeof(float) * (size_t)m.vertices);
-    L.halo = o;
-    o = align16(o + sizeof(int) * (size_t)m.halo);
-    L.f01 = o;
-    if (spt >= 5) o += 4 * slots;
-    L.f2 = o;
-    if (spt >= 5) o = align16(o + 2 * slots);
-    L.slo = o;
-    if (spt >= 6) o += sizeof(float2) * slots;
-    L.total = align16(o);
-    return L;
-}
-
 }  // namespace
 
 size_t persistent_flag_bytes(int npatch) { return flag_bytes(npatch); }
@@ -474,16 +420,7 @@ cudaError_t launch_persistent(const DevMesh &m, const DevState &s, const StepArg
             void *fn = persistent_kernel(g.plan.slots_per_thread, a.nonlinear_h, g.plan.cached, extra);
             if (!fn) return cudaErrorInvalidValue;
             PArgs P = make_pargs(m, s, a, M, parity, g.mx);
-            const SeLayout L = se_layout(g.mx, g.plan.slots_per_thread, g.plan.cached);
-            P.off_flux = (int)L.flux;
-            P.off_dummy = (int)L.dummy;
-            P.off_inv = (int)L.inv;
-            P.off_halo = (int)L.halo;
-            P.off_f01 = (int)L.f01;
-            P.off_f2 = (int)L.f2;
-            P.off_slo = (int)L.slo;
-            P.row_quads = L.quads;
-            P.row_vertices = g.mx.vertices;
+            set_layout(P, se_layout(g.mx, g.plan.slots_per_thread, g.plan.cached), g.mx);
             P.pack_first = g.first;
             P.pack_last = g.last;
             P.nsteps = nsteps;

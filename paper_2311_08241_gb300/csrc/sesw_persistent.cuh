@@ -67,9 +67,10 @@ struct PArgs {
     StepArgs a;
     int M, npatch;
     int nsteps;                  // baroclinic steps of this launch (k_persistent)
+    int npb;                     // patches of the pack (launches of one pack)
     unsigned tmem_cols;          // tensor-memory columns of a block (k_persistent, a power of two)
     int row_quads, row_vertices; // k_persistent: 16-byte quads of a vertex's row of fluxes; vertices per quad array
-    int off_dummy, off_f01, off_f2, off_slo;   // k_persistent: see SeLayout
+    int off_dummy, off_f01, off_f2, off_slo, off_hist;   // k_persistent: see SeLayout
     int team_threads, team_smem; // threads and shared-memory bytes of each patch of a block (k_persistent)
     // shared-memory carve-up (CACHED), in bytes from the dynamic shared base
     int off_flux, off_g, off_c, off_r, off_l, off_off, off_csr, off_inv, off_halo;
@@ -207,6 +208,24 @@ __device__ __forceinline__ void tmem_st4(uint32_t t, float a, float b, float c, 
                  : "memory");
 }
 
+constexpr int kMaxTeams = 4;
+
+
+// Barrier `bar` (1 ..) of a team of T threads (whole warps); barrier 0 is the block's.
+__device__ __forceinline__ void team_sync(int bar, int T)
+{
+    asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(T) : "memory");
+}
+
+// Shared-memory address of a flux place (21 bits of HostMesh::slot_f); corners that are not own
+// vertices write to the lane's dummy word.
+__device__ __forceinline__ uint32_t flux_place(const PArgs &P, uint32_t team, uint32_t dummy, uint32_t e)
+{
+    return e == 0x1fffffu ? dummy
+                          : team + (uint32_t)P.off_flux +
+                                16u * (((e & 15u) >> 2) * (uint32_t)P.row_vertices + (e >> 4)) + 4u * (e & 3u);
+}
+
 // A slot's static data: gradients, step coefficients (DevMesh::slot_k), forcing, and the
 // shared-memory addresses of its corners' elevations and of the places of its three fluxes.
 struct SlotData {
@@ -246,6 +265,20 @@ __device__ __forceinline__ void tmem_ld10(uint32_t t8, uint32_t t2, SlotData &q,
                  : "=f"(q.g.x), "=f"(q.g.y), "=f"(q.g.z), "=f"(q.g.w), "=f"(q.c.x), "=f"(q.c.y), "=f"(q.c.z),
                    "=f"(q.c.w), "=r"(l01), "=r"(l2)
                  : "r"(t8), "r"(t2));
+}
+
+// Words 4, 2, 2 and 1 of a thread at four places, waited for (a streamed SESM slot's state).
+__device__ __forceinline__ void tmem_ld9(uint32_t t4, uint32_t t2, uint32_t p2, uint32_t p1, float *f6, uint32_t &a,
+                                         uint32_t &b, uint32_t &c)
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%9];\n"
+                 "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%4, %5}, [%10];\n"
+                 "tcgen05.ld.sync.aligned.32x32b.x2.b32 {%6, %7}, [%11];\n"
+                 "tcgen05.ld.sync.aligned.32x32b.x1.b32 {%8}, [%12];\n"
+                 "tcgen05.wait::ld.sync.aligned;"
+                 : "=f"(f6[0]), "=f"(f6[1]), "=f"(f6[2]), "=f"(f6[3]), "=f"(f6[4]), "=f"(f6[5]), "=r"(a), "=r"(b),
+                   "=r"(c)
+                 : "r"(t4), "r"(t2), "r"(p2), "r"(p1));
 }
 
 __device__ __forceinline__ void tmem_ld8(uint32_t t8, SlotData &q)
@@ -524,6 +557,7 @@ inline PArgs make_pargs(const DevMesh &m, const DevState &s, const StepArgs &a, 
     P.a = a;
     P.M = M;
     P.nsteps = 1;
+    P.npb = 0;
     P.tmem_cols = 0;
     P.team_threads = P.team_smem = 0;
     P.npatch = m.npatch;
@@ -546,6 +580,71 @@ inline PArgs make_pargs(const DevMesh &m, const DevState &s, const StepArgs &a, 
     P.pack_first = 0;
     P.pack_last = 0;
     return P;
+}
+
+// Shared memory of one team, from its largest patch: elevation of own and halo vertices; the
+// fluxes, then 32 dummy words; 1/A_v and halo ids; from 5 slots per thread the flux places, from
+// 6 the low parts of the compensated sums. Vertex-major fluxes (cached): each own vertex has a row
+// of one word per incidence (4 words per quad, quad k of all vertices in array k), which the
+// element pass fills and the vertex pass reads 16 bytes at a time, in the place of an
+// index row and eight dependent 4-byte reads (the reads' bank conflicts kept the
+// shared-memory pipe busy longer than the element pass). Not cached: three words per slot.
+struct SeLayout {
+    size_t flux, dummy, inv, halo, f01, f2, slo, hist, total;
+    int quads;
+};
+
+inline SeLayout se_layout(const PatchMax &m, int spt, int cached)
+{
+    SeLayout L{};
+    const size_t slots = ((size_t)m.slots + 31) & ~(size_t)31;   // whole warps
+    size_t o = align16(sizeof(float) * (size_t)m.local);
+    L.flux = o;
+    if (!cached) {
+        L.total = align16(o + 12 * slots);
+        return L;
+    }
+    L.quads = std::max(2, (m.deg + 3) / 4);
+    o += 16 * (size_t)L.quads * (size_t)m.vertices;
+    L.dummy = o;
+    o += 128;
+    L.inv = o;
+    o = align16(o + sizeof(float) * (size_t)m.vertices);
+    L.halo = o;
+    o = align16(o + sizeof(int) * (size_t)m.halo);
+    L.f01 = o;
+    if (spt >= 5) o += 4 * slots;
+    L.f2 = o;
+    if (spt >= 5) o = align16(o + 2 * slots);
+    L.slo = o;
+    if (spt >= 6) o += sizeof(float2) * slots;
+    L.total = align16(o);
+    return L;
+}
+
+// The SESM teams: elevation (eta_AM) of own and halo vertices, fluxes, vertices' data as above, the
+// three levels of elevation that each own vertex keeps, and U_AB of the slots.
+inline SeLayout sesm_layout(const PatchMax &m)
+{
+    SeLayout L = se_layout(m, 1, 1);
+    L.hist = L.total;
+    L.slo = align16(L.hist + 3 * sizeof(float) * (size_t)m.vertices);
+    L.total = L.slo + sizeof(float2) * (((size_t)m.slots + 31) & ~(size_t)31);
+    return L;
+}
+
+inline void set_layout(PArgs &P, const SeLayout &L, const PatchMax &m)
+{
+    P.off_flux = (int)L.flux;
+    P.off_dummy = (int)L.dummy;
+    P.off_inv = (int)L.inv;
+    P.off_halo = (int)L.halo;
+    P.off_f01 = (int)L.f01;
+    P.off_f2 = (int)L.f2;
+    P.off_slo = (int)L.slo;
+    P.off_hist = (int)L.hist;
+    P.row_quads = L.quads;
+    P.row_vertices = m.vertices;
 }
 
 }  // namespace

@@ -19,9 +19,9 @@ namespace {
 // in registers; a vertex keeps eta^m, eta^{m-1}, eta^{m-2} in the registers of the thread
 // that updates it. The element pass needs only eta_AM at the corners, so the owner of a
 // vertex forms eta_AM^{m+1} right after eta^{m+1} and exchanges that one value, with the
-// same tagged words as the SE kernel (tag base + m for substep m, m = 1 .. M). As in the SE
-// kernel, the halo words of a thread's last-round slot are requested after its first round.
-constexpr int kSesmThreads = 384;   // registers: 65536 / (2 x 384) = 85 per thread
+// same tagged words as the SE kernel (tag base + x for substep x = 1 .. n M of a launch of n
+// steps; a launch loads the patch once for all of them).
+constexpr int kSesmThreads = 384;         // two blocks per SM; registers: 65536 / (2 x 384) = 85 per thread
 constexpr int kSesmVpt = 2;         // own vertices per thread at most
 
 template <int SPT, int NONLIN>
@@ -102,28 +102,29 @@ __global__ void __launch_bounds__(kSesmThreads, 2) k_persistent_sesm(PArgs P)
         u2[j] = u1[j];
         u1[j] = u0;
     };
-    auto halo_of = [&](unsigned l) { return (int)l < nown ? -1 : s_halo[l - nown]; };
-
     const int npre = nint >= T ? (nint / T) * T : nint;
-    // the last round's slot, when it is not a whole-round interior one: its halo words are
-    // requested right after the first round
-    const int ilast = threadIdx.x + (SPT - 1) * T;
-    const bool early = SPT > 1 && ilast >= npre && ilast < ns;
-    // one thread per halo vertex requests its tagged word before the interior rounds and stores
-    // the value after the eta_AM of the own vertices; the other slots then read every corner
-    // from shared memory (patches with more halo vertices than threads keep the reads per slot)
-    const bool hpre = nhalo <= T;
-    for (int m = 0; m <= P.M; m++) {
+    // One thread per halo vertex requests its tagged word before the interior rounds and stores
+    // the value after them; the other slots follow a barrier. x counts the substeps of the launch
+    // (the exchange's tags), m those of the running step, whose closing pass (m = M) is the momentum
+    // update of its last substep.
+    const int total = P.M * P.nsteps;
+    for (int x = 0, m = 0; x <= total; m++) {
         const bool vertex = m < P.M;
         if (m == 0) {
-            // no momentum update: U_AB^0 from level 0 and its aliases
+            // no momentum update: U_AB^0 from level 0 and its aliases; the sums start
 #pragma unroll
             for (int j = 0; j < SPT; j++) {
                 const int i = threadIdx.x + j * T;
+                shi[j] = make_float2(0.0f, 0.0f);
+                slo[j] = make_float2(0.0f, 0.0f);
+                u2[j] = u1[j];
                 if (i < ns) transport(j, i, u1[j], u1[j], u1[j], s_g[i], s_c[i].x);
             }
-        } else if (hpre) {
-            const unsigned long long *xs = P.xb[m & 1];
+#pragma unroll
+            for (int k = 0; k < kSesmVpt; k++) eh1[k] = eh2[k] = eh0[k];
+        } else {
+            const unsigned long long *xs = P.xb[x & 1];
+            const unsigned tag = base + (unsigned)x;
             const int hv = (int)threadIdx.x < nhalo ? s_halo[threadIdx.x] : -1;
             const unsigned long long hw = hv >= 0 ? ld_relaxed_gpu_u64(xs + hv) : 0ull;
 #pragma unroll
@@ -134,7 +135,11 @@ __global__ void __launch_bounds__(kSesmThreads, 2) k_persistent_sesm(PArgs P)
                     slot(j, i, sem[l.x], sem[l.y], sem[l.z], vertex);
                 }
             }
-            if (hv >= 0) sem[nown + threadIdx.x] = halo_eta(P, xs, hv, hw, base + (unsigned)m, abort_val, ok);
+            if (hv >= 0) sem[nown + threadIdx.x] = halo_eta(P, xs, hv, hw, tag, abort_val, ok);
+            for (int k = threadIdx.x + T; k < nhalo; k += T) {
+                const int v = s_halo[k];
+                sem[nown + k] = halo_eta(P, xs, v, ld_relaxed_gpu_u64(xs + v), tag, abort_val, ok);
+            }
             __syncthreads();
 #pragma unroll
             for (int j = 0; j < SPT; j++) {
@@ -145,57 +150,21 @@ __global__ void __launch_bounds__(kSesmThreads, 2) k_persistent_sesm(PArgs P)
                 }
             }
             if (!ok) s_abort = 1;
-        } else {
-            const unsigned tag = base + (unsigned)m;
-            const unsigned long long *xs = P.xb[m & 1];
-            unsigned long long q0 = 0ull, q1 = 0ull, q2 = 0ull;
-#pragma unroll
-            for (int j = 0; j < SPT; j++) {
-                const int i = threadIdx.x + j * T;
-                if (SPT > 1 && j == SPT - 1) {
-                    if (early) {
-                        const ushort4 l = s_l[i];
-                        const int h0 = halo_of(l.x), h1 = halo_of(l.y), h2 = halo_of(l.z);
-                        const float e0 = h0 < 0 ? sem[l.x] : halo_eta(P, xs, h0, q0, tag, abort_val, ok);
-                        const float e1 = h1 < 0 ? sem[l.y] : halo_eta(P, xs, h1, q1, tag, abort_val, ok);
-                        const float e2 = h2 < 0 ? sem[l.z] : halo_eta(P, xs, h2, q2, tag, abort_val, ok);
-                        slot(j, i, e0, e1, e2, vertex);
-                    } else if (i < npre) {
-                        const ushort4 l = s_l[i];
-                        slot(j, i, sem[l.x], sem[l.y], sem[l.z], vertex);
-                    }
-                } else if (i < ns) {
-                    const ushort4 l = s_l[i];
-                    if (i < npre) {
-                        slot(j, i, sem[l.x], sem[l.y], sem[l.z], vertex);
-                    } else {
-                        const int h0 = halo_of(l.x), h1 = halo_of(l.y), h2 = halo_of(l.z);
-                        const unsigned long long w0 = h0 < 0 ? 0ull : ld_relaxed_gpu_u64(xs + h0);
-                        const unsigned long long w1 = h1 < 0 ? 0ull : ld_relaxed_gpu_u64(xs + h1);
-                        const unsigned long long w2 = h2 < 0 ? 0ull : ld_relaxed_gpu_u64(xs + h2);
-                        const float e0 = h0 < 0 ? sem[l.x] : halo_eta(P, xs, h0, w0, tag, abort_val, ok);
-                        const float e1 = h1 < 0 ? sem[l.y] : halo_eta(P, xs, h1, w1, tag, abort_val, ok);
-                        const float e2 = h2 < 0 ? sem[l.z] : halo_eta(P, xs, h2, w2, tag, abort_val, ok);
-                        slot(j, i, e0, e1, e2, vertex);
-                    }
-                }
-                if (j == 0 && early) {
-                    const ushort4 l = s_l[ilast];
-                    const int h0 = halo_of(l.x), h1 = halo_of(l.y), h2 = halo_of(l.z);
-                    if (h0 >= 0) q0 = ld_relaxed_gpu_u64(xs + h0);
-                    if (h1 >= 0) q1 = ld_relaxed_gpu_u64(xs + h1);
-                    if (h2 >= 0) q2 = ld_relaxed_gpu_u64(xs + h2);
-                }
-            }
-            if (!ok) s_abort = 1;
         }
-        if (!vertex) break;
+        if (!vertex) {
+            if (x == total) break;
+            m = -1;               // the next step starts at the same x; its first pass reads no halo
+            __syncthreads();
+            if (s_abort) break;
+            continue;
+        }
         __syncthreads();
         if (s_abort) break;
+        x++;
 
         // vertex pass: eta^{m+1}, then eta_AM^{m+1} for the own slots and the neighbours
-        unsigned long long *xout = P.xb[(m + 1) & 1];
-        const unsigned long long tag_out = (unsigned long long)(base + (unsigned)(m + 1)) << 32;
+        unsigned long long *xout = P.xb[x & 1];
+        const unsigned long long tag_out = (unsigned long long)(base + (unsigned)x) << 32;
         const bool publish = p != a.silent_patch;
         bool bad = false;
 #pragma unroll
@@ -237,8 +206,269 @@ __global__ void __launch_bounds__(kSesmThreads, 2) k_persistent_sesm(PArgs P)
     }
     if (threadIdx.x == 0 && atomicAdd(exit_count, 1u) == gridDim.x - 1) {
         *exit_count = 0u;
-        *base_word = base + (unsigned)P.M + 1u;
+        *base_word = base + (unsigned)total + 1u;
     }
+}
+
+// ---------------------------------------------------------------------------------
+// The same for larger patches (up to 7 slots per thread): one block per SM holds one to four
+// teams, each with its own patch, with the flux rows and tensor memory of the SE kernel
+// (sesw_persistent.cu). U^{m-1} of a slot lives in registers, U_AB^{m-1} in shared memory, U^{m-2}, the
+// sum and the packed addresses (9 words) in tensor memory; the static data (40 B per slot and
+// substep) come from L2. Before, all state streamed from L2 as well (k_persistent_sesm_stream, now
+// for patches beyond this): 408k vertices, two steps, 1003 -> 654 us.
+// (On-chip patches stay with k_persistent_sesm: teams with their static data in tensor memory measured
+// the same, 488 against 490 us for four steps of the 200k-vertex channel.)
+constexpr int kSesmTeamThreads = 1024;   // 64 registers per thread
+
+// A thread's words in tensor memory: the sums (4 per slot), then U^{m-2} (2), then the
+// addresses of the three corners and three flux places as 16-bit word indices (2 and 1).
+template <int SPT>
+struct SesmState {
+    __device__ static __forceinline__ void store(uint32_t tm, int j, float2 hi, float2 lo, float2 u)
+    {
+        tmem_st4(tm + 4 * j, hi.x, hi.y, lo.x, lo.y);
+        tmem_st2(tm + 4 * SPT + 2 * j, __float_as_uint(u.x), __float_as_uint(u.y));
+    }
+    __device__ static __forceinline__ void store_places(uint32_t tm, int j, const SlotData &q)
+    {
+        tmem_st2(tm + 6 * SPT + 2 * j, (q.a0 >> 2) | (q.a1 << 14), (q.a2 >> 2) | (q.f0 << 14));
+        asm volatile("tcgen05.st.sync.aligned.32x32b.x1.b32 [%0], {%1};" ::"r"(tm + 8 * SPT + j),
+                     "r"((q.f1 >> 2) | (q.f2 << 14))
+                     : "memory");
+    }
+    __device__ static __forceinline__ void load(uint32_t tm, int j, float2 &hi, float2 &lo, float2 &u, SlotData &q)
+    {
+        float st[6];
+        uint32_t p0, p1, p2;
+        tmem_ld9(tm + 4 * j, tm + 4 * SPT + 2 * j, tm + 6 * SPT + 2 * j, tm + 8 * SPT + j, st, p0, p1, p2);
+        hi = make_float2(st[0], st[1]);
+        lo = make_float2(st[2], st[3]);
+        u = make_float2(st[4], st[5]);
+        q.a0 = (p0 & 0xffffu) * 4u;
+        q.a1 = (p0 >> 16) * 4u;
+        q.a2 = (p1 & 0xffffu) * 4u;
+        q.f0 = (p1 >> 16) * 4u;
+        q.f1 = (p2 & 0xffffu) * 4u;
+        q.f2 = (p2 >> 16) * 4u;
+    }
+};
+
+// Tensor-memory words of a thread.
+__host__ __device__ constexpr int sesm_words(int spt) { return (9 * spt + 3) & ~3; }
+
+template <int SPT, int NONLIN>
+__device__ __forceinline__ void sesm_patch(const PArgs &P, const int p, const int pack, const int npb,
+                                           const uint32_t tm, unsigned char *smem_raw, int &s_abort, const int tid,
+                                           const int T, const int bar)
+{
+    using SS = SesmState<SPT>;
+    const uint32_t team = (uint32_t)__cvta_generic_to_shared(smem_raw);
+    const int wbase = __shfl_sync(0xffffffffu, tid & ~31, 0);   // the warp's first thread
+    const int s0 = P.patch_slot[p], ns = P.patch_slot[p + 1] - s0;
+    const int nsp = (ns + 31) & ~31;    // slots of whole warps
+    const int nown_s = P.patch_own[p], nint = P.patch_int[p];
+    const int v0 = P.patch_v[p], nown = P.patch_v[p + 1] - v0;
+    const int hb = P.patch_halo[p], nhalo = P.patch_halo[p + 1] - hb;
+    const StepArgs a = P.a;
+    const float dt = P.patch_dt[p];
+    unsigned *base_word = P.flags + (size_t)(1 + 2 * pack) * kFlagStride;
+    unsigned *exit_count = base_word + kFlagStride;
+    const unsigned base = ld_relaxed_gpu(base_word);
+    const unsigned abort_val = base + 1u == 0u ? 1u : base + 1u;   // never 0, unique per launch
+
+    float *sem = reinterpret_cast<float *>(smem_raw);   // eta_AM of the own vertices, then of the halo
+    float *s_inv = reinterpret_cast<float *>(smem_raw + P.off_inv);
+    int *s_halo = reinterpret_cast<int *>(smem_raw + P.off_halo);
+    float *hist = reinterpret_cast<float *>(smem_raw + P.off_hist);   // three levels of row_vertices each
+    {
+        float4 *rows = reinterpret_cast<float4 *>(smem_raw + P.off_flux);
+        for (int i = tid; i < P.row_quads * P.row_vertices; i += T) rows[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    }
+    for (int i = tid; i < nown; i += T) {
+        s_inv[i] = P.inv_av[v0 + i];
+        hist[i] = P.eta_in[v0 + i];
+    }
+    for (int i = tid; i < nhalo; i += T) s_halo[i] = P.halo_v[hb + i];
+    if (tid == 0) s_abort = 0;
+    // threads without a slot in their last round hold an all-zero one (see k_persistent)
+    const uint32_t dummy = team + (uint32_t)P.off_dummy + 4u * (tid & 31);
+    const uint32_t uab_at = team + (uint32_t)P.off_slo;      // U_AB^{m-1} of the slots
+    float2 u1[SPT];
+#pragma unroll
+    for (int j = 0; j < SPT; j++) {
+        const int i = tid + j * T;
+        const bool in = i < ns;
+        const int s = s0 + (in ? i : 0);
+        const ushort4 l = P.sl[s];
+        const uint2 f = in ? P.sf[s] : make_uint2(0xffffffffu, 0x7fffffffu);
+        SlotData q;
+        q.a0 = team + 4u * l.x;
+        q.a1 = team + 4u * l.y;
+        q.a2 = team + 4u * l.z;
+        q.f0 = flux_place(P, team, dummy, f.x & 0x1fffffu);
+        q.f1 = flux_place(P, team, dummy, (f.x >> 21) | ((f.y & 0x3ffu) << 11));
+        q.f2 = flux_place(P, team, dummy, (f.y >> 10) & 0x1fffffu);
+        SS::store_places(tm, j, q);
+        u1[j] = in ? P.U[s] : make_float2(0.0f, 0.0f);
+    }
+    tmem_wait_st();
+    team_sync(bar, T);
+
+    // Slots [lo, hi) (multiples of 32, whole warps) at substep ms of the step: the momentum update (ms > 0),
+    // then (vertex) U_AB, its fluxes and the compensated sum. At ms = 0 every earlier level is level 0
+    // and the sum starts.
+    auto elements = [&](int lo, int hi, int ms, bool vertex) {
+#pragma unroll
+        for (int j = 0; j < SPT; j++) {
+            const int w = wbase + j * T;
+            if (w >= lo && w < hi) {
+                const int i = tid + j * T;
+                SlotData q;
+                float2 v2, hi2, lo2;
+                const int s = s0 + min(i, ns - 1);
+                q.g = __ldg(P.sg + s);
+                q.c = __ldg(P.sc + s);
+                q.r = __ldg(P.R + s);
+                SS::load(tm, j, hi2, lo2, v2, q);
+                if (i >= ns) {
+                    q.g = q.c = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                    q.r = make_float2(0.0f, 0.0f);
+                }
+                float2 u0 = u1[j], up = u1[j];
+                if (ms > 0) {
+                    const float e0 = lds(q.a0), e1 = lds(q.a1), e2 = lds(q.a2);
+                    u0 = sesm_momentum<NONLIN>(e0, e1, e2, q.g, q.c.y, a.g, q.c.z, dt, q.r, up,
+                                               lds2(uab_at + 8 * i));
+                } else {
+                    v2 = u0;
+                    hi2 = lo2 = make_float2(0.0f, 0.0f);
+                }
+                u1[j] = u0;
+                if (vertex) {
+                    const float2 F = sesm_ab3(u0, up, v2, a.ab0, a.ab1, a.ab2);
+                    two_sum_acc2<0>(hi2, lo2, F);
+                    float f3[3];
+                    corner_fluxes<0>(F, q.g, __fmul_rn(dt, q.c.x), f3);
+                    sts(q.f0, f3[0]);
+                    sts(q.f1, f3[1]);
+                    sts(q.f2, f3[2]);
+                    sts2(uab_at + 8 * i, F);
+                    SS::store(tm, j, hi2, lo2, up);    // U^{m-1} of this substep is U^{m-2} of the next
+                }
+            }
+        }
+        tmem_wait_st();
+    };
+
+    bool ok = true;
+    const int npre = nint >= T ? (nint / T) * T : nint & ~31;
+    // x counts the substeps of the launch (the exchange's tags); ms those of the running step, whose
+    // closing pass (ms = M) is the momentum update of its last substep
+    const int total = P.M * P.nsteps;
+    int cur = 0;                      // level of hist with eta^m
+    for (int x = 0, ms = 0; x <= total; ms++) {
+        const bool vertex = ms < P.M;
+        if (ms == 0) {
+            elements(0, nsp, 0, true);
+        } else {
+            const unsigned long long *xs = P.xb[x & 1];
+            const unsigned tag = base + (unsigned)x;
+            const int hv = tid < nhalo ? s_halo[tid] : -1;
+            const unsigned long long hw = hv >= 0 ? ld_relaxed_gpu_u64(xs + hv) : 0ull;
+            elements(0, npre, ms, vertex);
+            if (hv >= 0) sem[nown + tid] = halo_eta(P, xs, hv, hw, tag, abort_val, ok);
+            for (int k = tid + T; k < nhalo; k += T) {
+                const int v = s_halo[k];
+                sem[nown + k] = halo_eta(P, xs, v, ld_relaxed_gpu_u64(xs + v), tag, abort_val, ok);
+            }
+            team_sync(bar, T);
+            elements(npre, nsp, ms, vertex);
+            if (!ok) s_abort = 1;
+        }
+        if (!vertex) {
+            if (x == total) break;
+            ms = -1;                  // the next step starts at the same x; its first pass reads no halo
+            team_sync(bar, T);
+            if (s_abort) break;
+            continue;
+        }
+        team_sync(bar, T);
+        if (s_abort) break;
+
+        // vertex pass: eta^{m+1}, then eta_AM^{m+1} for the own slots and the neighbours
+        x++;
+        unsigned long long *xout = P.xb[x & 1];
+        const unsigned long long tag_out = (unsigned long long)(base + (unsigned)x) << 32;
+        const bool publish = p != a.silent_patch;
+        const int nv = P.row_vertices, nxt = cur == 2 ? 0 : cur + 1, prv = cur == 0 ? 2 : cur - 1;
+        bool bad = false;
+        for (int i = tid; i < nown; i += T) {
+            float sum = 0.0f;
+            uint32_t row = team + (uint32_t)P.off_flux + 16u * (uint32_t)i;
+            for (int k = 0; k < P.row_quads; k++, row += 16u * (uint32_t)nv) {
+                const float4 c = lds4(row);
+                sum = __fadd_rn(__fadd_rn(__fadd_rn(__fadd_rn(sum, c.x), c.y), c.z), c.w);
+            }
+            const float h0 = hist[cur * nv + i];
+            const float h1 = ms == 0 ? h0 : hist[prv * nv + i], h2 = ms == 0 ? h0 : hist[nxt * nv + i];
+            float e = vertex_eta(h0, sum, s_inv[i]);
+            if (P.W) e = __fmaf_rn(-dt, __ldg(P.W + v0 + i), e);
+            const float em = sesm_am4(e, h0, h1, h2, a.am0, a.am1, a.am2, a.am3);
+            hist[nxt * nv + i] = e;
+            if (ms == 0) hist[prv * nv + i] = h0;
+            sem[i] = em;
+            if (publish) st_relaxed_gpu_u64(xout + v0 + i, tag_out | __float_as_uint(em));
+            bad |= !(fabsf(e) <= a.eta_bound);
+        }
+        cur = nxt;
+        if (bad) atomicOr(P.status, 1u);
+        team_sync(bar, T);
+    }
+    team_sync(bar, T);
+
+    for (int i = tid; i < nown; i += T) P.eta_out[v0 + i] = hist[cur * P.row_vertices + i];
+#pragma unroll
+    for (int j = 0; j < SPT; j++) {
+        const int i = tid + j * T;
+        SlotData q;
+        float2 hi2, lo2, u;
+        SS::load(tm, j, hi2, lo2, u, q);
+        if (i < ns) {
+            P.U[s0 + i] = u1[j];
+            if (i < nown_s) {
+                const int w = P.sv[s0 + i].w;
+                P.Umean[w] = make_float2((hi2.x + lo2.x) * a.inv_M, (hi2.y + lo2.y) * a.inv_M);
+            }
+        }
+        __syncwarp();
+    }
+    if (tid == 0 && atomicAdd(exit_count, 1u) == (unsigned)npb - 1u) {
+        *exit_count = 0u;
+        *base_word = base + (unsigned)total + 1u;
+    }
+}
+
+template <int SPT, int NONLIN>
+__global__ void __launch_bounds__(kSesmTeamThreads, 1) k_persistent_sesm_teams(PArgs P)
+{
+    extern __shared__ __align__(16) unsigned char smem_all[];
+    __shared__ uint32_t s_tmem;
+    __shared__ int s_abort[kMaxTeams];
+    const int warp = threadIdx.x >> 5;
+    if (warp == 0) tmem_alloc(&s_tmem, P.tmem_cols);
+    __syncthreads();
+    tmem_fence_after_sync();
+    const uint32_t base = s_tmem;
+    const uint32_t tm = base + ((uint32_t)(warp & 3) << 21) + (uint32_t)((warp >> 2) * sesm_words(SPT));
+    const int T = P.team_threads, team = (int)threadIdx.x / T, tid = (int)threadIdx.x - team * T;
+    const int npb = P.npb, q = (int)blockIdx.x + team * (int)gridDim.x;
+    if (q < npb)
+        sesm_patch<SPT, NONLIN>(P, P.pack_patch[P.pack_base + q], P.pack_index, npb, tm,
+                                smem_all + (size_t)team * P.team_smem, s_abort[team], tid, T, team + 1);
+    tmem_fence_before_sync();
+    __syncthreads();
+    if (warp == 0) tmem_dealloc(base, P.tmem_cols);
 }
 
 void *sesm_kernel(int spt, int nonlin)
@@ -248,6 +478,17 @@ void *sesm_kernel(int spt, int nonlin)
     case 2: return nonlin ? (void *)k_persistent_sesm<2, 1> : (void *)k_persistent_sesm<2, 0>;
     case 3: return nonlin ? (void *)k_persistent_sesm<3, 1> : (void *)k_persistent_sesm<3, 0>;
     case 4: return nonlin ? (void *)k_persistent_sesm<4, 1> : (void *)k_persistent_sesm<4, 0>;
+    default: return nullptr;
+    }
+}
+
+void *sesm_teams_kernel(int spt, int nonlin)
+{
+    switch (spt) {
+    case 4: return nonlin ? (void *)k_persistent_sesm_teams<4, 1> : (void *)k_persistent_sesm_teams<4, 0>;
+    case 5: return nonlin ? (void *)k_persistent_sesm_teams<5, 1> : (void *)k_persistent_sesm_teams<5, 0>;
+    case 6: return nonlin ? (void *)k_persistent_sesm_teams<6, 1> : (void *)k_persistent_sesm_teams<6, 0>;
+    case 7: return nonlin ? (void *)k_persistent_sesm_teams<7, 1> : (void *)k_persistent_sesm_teams<7, 0>;
     default: return nullptr;
     }
 }
@@ -302,34 +543,95 @@ PersistentPlan persistent_plan_sesm(const PatchMax &m, int blocks_per_sm)
     return plan;
 }
 
+PersistentPlan persistent_plan_sesm_teams(const PatchMax &m, int blocks_per_sm)
+{
+    PersistentPlan plan;
+    int dev = 0, smem_optin = 0, smem_sm = 0, nsm = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess) {
+        cudaGetLastError();
+        return plan;
+    }
+    if (m.deg > 16) return plan;   // HostMesh::slot_f
+    const int teams = std::min(std::max(blocks_per_sm, 1), kMaxTeams);
+    const int max_threads = kSesmTeamThreads / teams / 32 * 32;
+    if (smem_optin < 2048 || smem_sm < 4096) return plan;
+    const size_t budget = std::min((size_t)smem_optin - 1024, (size_t)smem_sm - 2048);
+    for (int spt = 4; spt <= 7; spt++) {
+        const int t = std::max(32, ((m.slots + spt - 1) / spt + 31) / 32 * 32);
+        if (t > max_threads) continue;
+        const unsigned cols = tmem_columns(teams * t, sesm_words(spt));
+        const size_t team_smem = sesm_layout(m).total;
+        const size_t smem = std::max(teams * team_smem, tmem_smem_floor(cols, (size_t)smem_sm));
+        if (smem > budget || cols > 512u) return plan;
+        for (int nonlin = 0; nonlin < 2; nonlin++) {
+            void *fn = sesm_teams_kernel(spt, nonlin);
+            int occ = 0;
+            if (!fn || raise_smem_limit(fn) < (int)smem ||
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, teams * t, smem) != cudaSuccess || occ < 1) {
+                cudaGetLastError();
+                return plan;
+            }
+        }
+        plan.slots_per_thread = spt;
+        plan.threads = t;
+        plan.cached = 1;
+        plan.stream = 1;
+        plan.blocks_per_sm = blocks_per_sm;
+        plan.teams = teams;
+        plan.team_smem = (int)team_smem;
+        plan.tmem_cols = (int)cols;
+        plan.grid = nsm;
+        plan.smem = smem;
+        return plan;
+    }
+    return plan;
+}
+
 cudaError_t persistent_prepare_sesm(const PersistentPlan &plan)
 {
     for (int nonlin = 0; nonlin < 2; nonlin++) {
-        void *fn = sesm_kernel(plan.slots_per_thread, nonlin);
+        void *fn = plan.teams ? sesm_teams_kernel(plan.slots_per_thread, nonlin)
+                              : sesm_kernel(plan.slots_per_thread, nonlin);
         if (!fn || raise_smem_limit(fn) < (int)plan.smem) return cudaErrorInvalidValue;
     }
     return cudaSuccess;
 }
 
-cudaError_t launch_persistent_sesm(const DevMesh &m, const DevState &s, const StepArgs &a, int M, int parity,
+cudaError_t launch_persistent_sesm(const DevMesh &m, const DevState &s, const StepArgs &a, int M, int parity, int nsteps,
                                    const std::vector<PackPlan> &packs, cudaStream_t stream)
 {
     // one cooperative launch per pack, each with its own plan, layout and tag base
     for (size_t k = 0; k < packs.size(); k++) {
         const PackPlan &pk = packs[k];
-        if (pk.plan_sesm.stream) {
+        const PersistentPlan &pl = pk.plan_sesm;
+        if (pl.stream && !pl.teams) {
+            if (nsteps != 1) return cudaErrorInvalidValue;   // one step per launch
             const cudaError_t e = launch_persistent_sesm_stream_pack(m, s, a, M, parity, pk, (int)k, stream);
             if (e != cudaSuccess) return e;
             continue;
         }
-        void *fn = sesm_kernel(pk.plan_sesm.slots_per_thread, a.nonlinear_h);
+        void *fn = pl.teams ? sesm_teams_kernel(pl.slots_per_thread, a.nonlinear_h)
+                            : sesm_kernel(pl.slots_per_thread, a.nonlinear_h);
         if (!fn) return cudaErrorInvalidValue;
         PArgs P = make_pargs(m, s, a, M, parity, pk.mx);
         P.pack_base = pk.base;
         P.pack_index = (int)k;
+        P.npb = pk.nblocks;
+        P.nsteps = nsteps;
+        int grid = pk.nblocks, threads = pl.threads;
+        if (pl.teams) {
+            set_layout(P, sesm_layout(pk.mx), pk.mx);
+            P.tmem_cols = (unsigned)pl.tmem_cols;
+            P.team_threads = pl.threads;
+            P.team_smem = pl.team_smem;
+            grid = std::min(pl.grid, pk.nblocks);
+            threads = pl.teams * pl.threads;
+        }
         void *args[] = {&P};
-        cudaError_t e =
-            cudaLaunchCooperativeKernel(fn, dim3(pk.nblocks), dim3(pk.plan_sesm.threads), args, pk.plan_sesm.smem, stream);
+        const cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(threads), args, pl.smem, stream);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
