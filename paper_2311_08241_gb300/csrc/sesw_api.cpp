@@ -773,6 +773,16 @@ static int upload_batch(sesw_ctx *c, const sesw_mesh *meshes, int n)
         }
         TRY(upload(c, &d.pack_patch, pp, "pack_patch"));
         TRY(upload(c, &d.pack_off_d, d.pack_off, "pack_off"));
+        if (n == 1 && packs.size() == 1 && !packs[0].plan.stream && c->blocks_per_sm == 0) {
+            std::vector<int> grp, halo;
+            std::vector<unsigned> readers;
+            d.cluster = sesw::cluster_plan(hm, packs[0].mx.deg, grp, readers, halo);
+            if (d.cluster.blocks > 0) {
+                TRY(upload(c, &d.cluster_grp, grp, "cluster_grp"));
+                TRY(upload(c, &d.cluster_readers, readers, "cluster_readers"));
+                TRY(upload(c, &d.cluster_halo, halo, "cluster_halo"));
+            }
+        }
     }
     {
         std::vector<int> bslot(hm.nbasin + 1);

@@ -94,6 +94,13 @@ int prepare_mesh(const sesw_mesh &m, int patch_vertices, HostMesh &out, std::str
 uint64_t hilbert2d(uint32_t x, uint32_t y, int bits);
 uint64_t hilbert3d(uint32_t x, uint32_t y, uint32_t z, int bits);
 
+// One cluster of blocks that advances a whole small mesh (k_cluster); blocks = 0: none.
+struct ClusterPlan {
+    int blocks = 0, threads = 0;
+    int own = 0, deg = 0;          // most own vertices of a block, most incidences of a vertex
+    size_t smem = 0;
+};
+
 // Device arrays of one prepared mesh plus the state.
 struct DevMesh {
     int nv = 0, ne = 0, npatch = 0, nslot = 0, max_patch_slots = 0;
@@ -145,6 +152,12 @@ struct DevMesh {
     ushort4 *slot_l = nullptr;
     uint2 *slot_f = nullptr;
     int max_patch_local = 0, max_patch_vertices = 0, max_patch_halo = 0, max_patch_csr = 0;
+    // small meshes: the cluster's plan, the patch ranges of its blocks, the blocks that read each vertex,
+    // the number of vertices that each block reads and does not own
+    ClusterPlan cluster;
+    int *cluster_grp = nullptr;
+    unsigned *cluster_readers = nullptr;
+    int *cluster_halo = nullptr;
 };
 
 struct DevState {
@@ -307,6 +320,14 @@ cudaError_t launch_slot_coef(const DevMesh &m, float g, cudaStream_t stream);
 // One launch per pack advances nsteps steps (1 where a pack runs k_persistent_sesm_stream).
 cudaError_t launch_persistent_sesm(const DevMesh &m, const DevState &s, const StepArgs &a, int M, int parity, int nsteps,
                                    const std::vector<PackPlan> &packs, cudaStream_t stream);
+
+// Small meshes: the cluster's plan (blocks 0 when the mesh is too large or no cluster fits), the patch
+// ranges of its blocks, the blocks that read each vertex, and how many vertices each block reads
+// without owning them. deg: most incidences of a vertex.
+ClusterPlan cluster_plan(const HostMesh &hm, int deg, std::vector<int> &grp, std::vector<unsigned> &readers,
+                         std::vector<int> &halo);
+cudaError_t launch_cluster(const DevMesh &m, const DevState &s, const StepArgs &a, int M, int parity, int nsteps,
+                           cudaStream_t stream);
 
 struct Surrogate;
 void surrogate_release(sesw_ctx *c);

@@ -133,3 +133,27 @@ def test_slots_per_thread(S, nx, ny, bps, spt):
     got, info = _run(S, case.mesh, p, [2], PERSISTENT, bps=bps, form=1)
     assert info["slots_per_thread"] == spt and info["streamed"] == 0, info
     _same(ref, got, f"{spt} slots per thread")
+
+
+@pytest.mark.parametrize("nx,ny", [(16, 16), (17, 31), (23, 23), (40, 37), (60, 61), (66, 64)])
+@pytest.mark.parametrize("M,parts", [(1, [1]), (1, [2]), (2, [1, 3]), (9, [2])])
+def test_small_meshes_in_one_cluster(S, nx, ny, M, parts):
+    """The cluster of 8 or 16 blocks that takes small meshes (up to one slot per thread), from too few
+    patches for it to too many slots, with every optional term, against graph mode and against the
+    kernel that exchanges through L2 (an explicit residency)."""
+    mesh = I.tiny_jittered_case(nx=nx, ny=ny, seed=4).mesh
+    p = I.Params(tau=10.0 * M, M=M)
+    for extra in (False, True):
+        ref, _ = _run(S, mesh, p, [1] * sum(parts), GRAPH, extra=extra)
+        got, info = _run(S, mesh, p, parts, PERSISTENT, extra=extra)
+        assert info["mode"] == PERSISTENT
+        _same(ref, got, "cluster")
+        _same(ref, _run(S, mesh, p, parts, PERSISTENT, bps=2, extra=extra)[0], "through L2")
+
+
+def test_small_mesh_of_separate_parts(S):
+    """Disconnected fans: blocks of a cluster that read nothing from the others."""
+    mesh = _fan(6, 120)
+    p = I.Params(tau=20.0, M=5)
+    ref, _ = _run(S, mesh, p, [2], GRAPH)
+    _same(ref, _run(S, mesh, p, [2], PERSISTENT)[0], "fans")
