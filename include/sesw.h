@@ -289,8 +289,10 @@ int sesw_set_large_basins(sesw_ctx *ctx, int32_t blocks_per_sm, int32_t form);
  * sphere, is faster at 2). Takes effect at the next mesh upload. */
 int sesw_set_blocks_per_sm(sesw_ctx *ctx, int32_t blocks_per_sm);
 
-/* Threads per block of the substep kernel (a multiple of 32 in [32, 1024]);
- * default 256. Takes effect at the next advance. */
+/* Threads per block of the substep kernel (a multiple of 32 in [32, 1024]). Until it is
+ * called, graph mode takes 256 for SESM and for the SE scheme the size whose blocks need
+ * the fewest rounds of the slot loop over the whole device (results do not depend on it).
+ * Takes effect at the next advance. */
 int sesw_set_block_threads(sesw_ctx *ctx, int32_t threads);
 
 /* Validate, reorder and upload a mesh (mesh prep: geometry, space-filling-curve

@@ -115,6 +115,14 @@ int zalloc(sesw_ctx *c, T **dst, size_t n, const char *name)
         if (r_ != SESW_OK) return r_; \
     } while (0)
 
+// Threads per block of the graph mode's substep kernel.
+int graph_threads(const sesw_ctx *c)
+{
+    if (c->block_threads > 0) return c->block_threads;
+    if (!c->have_params || c->params.scheme == 1) return 256;
+    return sesw::substep_threads(c->dm, c->params.nonlinear_h != 0, c->visc_on);
+}
+
 int capture_step_graph(sesw_ctx *c, int parity, cudaGraphExec_t *out)
 {
     cudaGraph_t g = nullptr;
@@ -154,7 +162,7 @@ int capture_step_graph(sesw_ctx *c, int parity, cudaGraphExec_t *out)
             q.e2 = el(m - 2);
             q.e3 = el(m - 3);
             q.enew = el(m + 1);
-            e = sesw::launch_sesm(c->dm, c->ds, c->args, q, c->block_threads, c->cap_stream);
+            e = sesw::launch_sesm(c->dm, c->ds, c->args, q, graph_threads(c), c->cap_stream);
         }
         if (e == cudaSuccess) e = sesw::launch_step_epilogue(c->dm, c->ds, c->args, c->cap_stream);
         if (e == cudaSuccess && M % 5 != 0)
@@ -164,13 +172,14 @@ int capture_step_graph(sesw_ctx *c, int parity, cudaGraphExec_t *out)
         // with the barotropic viscosity each substep reads U^m from one buffer (its
         // neighbours' too) and writes U^{m+1} to the other; U^M goes back to ds.U
         int p = parity;
+        const int threads = graph_threads(c);
         float2 *B[2] = {c->ds.U, c->ds.U_x[0]};
         for (int m = 0; m < c->params.M && e == cudaSuccess; m++) {
             if (c->visc_on) {
                 sesw::SubstepViscArgs v{c->vargs, m == 0, B[m & 1], B[(m + 1) & 1]};
-                e = sesw::launch_substep(c->dm, c->ds, c->args, p, c->block_threads, c->cap_stream, &v);
+                e = sesw::launch_substep(c->dm, c->ds, c->args, p, threads, c->cap_stream, &v);
             } else {
-                e = sesw::launch_substep(c->dm, c->ds, c->args, p, c->block_threads, c->cap_stream);
+                e = sesw::launch_substep(c->dm, c->ds, c->args, p, threads, c->cap_stream);
             }
             p ^= 1;
         }
@@ -1411,7 +1420,7 @@ int sesw_get_info(sesw_ctx *c, sesw_info *info)
     info->patch_vertices = c->patch_vertices_used;
     // the persistent plan of the scheme in use (SE until SESM parameters are set)
     const sesw::PersistentPlan &pl = c->have_params && c->params.scheme == 1 ? c->plan_sesm : c->plan;
-    info->block_threads = c->mode == SESW_MODE_PERSISTENT ? pl.threads : c->block_threads;
+    info->block_threads = c->mode == SESW_MODE_PERSISTENT ? pl.threads : graph_threads(c);
     info->mode = c->mode;
     info->blocks_per_sm = c->mode == SESW_MODE_PERSISTENT ? pl.blocks_per_sm : 0;
     info->slots_per_thread = c->mode == SESW_MODE_PERSISTENT ? pl.slots_per_thread : 0;

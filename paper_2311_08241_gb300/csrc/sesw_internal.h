@@ -230,6 +230,7 @@ struct StepArgs {
 // launch error.
 cudaError_t launch_substep(const DevMesh &m, const DevState &s, const StepArgs &a, int parity,
                            int block, cudaStream_t stream, const SubstepViscArgs *visc = nullptr);
+int substep_threads(const DevMesh &m, bool nonlin, bool visc);
 cudaError_t substep_smem_attr(const DevMesh &m);
 cudaError_t launch_step_epilogue(const DevMesh &m, const DevState &s, const StepArgs &a,
                                  cudaStream_t stream);
@@ -387,7 +388,7 @@ struct sesw_ctx {
     void *user = nullptr;
     std::string err;
     int patch_vertices = 256;
-    int block_threads = 256;
+    int block_threads = 0;         // graph mode; 0 = chosen by substep_threads (SESM: 256)
     int mode_req = SESW_MODE_AUTO, mode = SESW_MODE_GRAPH;
     int blocks_per_sm = 0;         // persistent mode; 0 = try 2, then 1
     int form = SESW_FORM_AUTO;     // persistent mode: which kernel a pack runs (sesw_set_persistent_form)

@@ -35,6 +35,17 @@ struct ViscTables {
     const float2 *r2;
 };
 
+// One slot of the tables, loaded ahead of its use.
+struct ViscRow {
+    int4 q, c;
+    float4 a, b;
+};
+
+__device__ __forceinline__ ViscRow visc_row(const ViscTables &T, int s)
+{
+    return ViscRow{T.q[s], T.c[s], T.a[s], T.b[s]};
+}
+
 // Barotropic viscous regularisation, Eq. (viscosity_BT), of slot s (depth H, transport
 // Us, corner elevations e[3], area A_e): a two-point flux across each edge k (corners k
 // and k+1) with a neighbour,
@@ -45,12 +56,13 @@ struct ViscTables {
 // opposite corner when nonlinear). Neighbours are read from their owner slots, so every
 // copy of an element computes the same value.
 template <int ROT>
-__device__ __forceinline__ float2 visc_of(int s, float H, float2 Us, const float e[3], float area, const ViscTables T,
-                                          const float2 *U, const float *__restrict__ eta, const ViscArgs va)
+__device__ __forceinline__ float2 visc_of(int s, float H, float2 Us, const float e[3], float area, const ViscTables &T,
+                                          const ViscRow &row, const float2 *U, const float *__restrict__ eta,
+                                          const ViscArgs va)
 {
     const float ux = Us.x / H, uy = Us.y / H;
-    const int4 tq = T.q[s], tc = T.c[s];
-    const float4 ta = T.a[s], tb = T.b[s];
+    const int4 tq = row.q, tc = row.c;
+    const float4 ta = row.a, tb = row.b;
     const int q[3] = {tq.x, tq.y, tq.z};
     const int oc[3] = {tc.x, tc.y, tc.z};
     const float h0[3] = {__int_as_float(tq.w), __int_as_float(tc.w), ta.w};
@@ -129,23 +141,35 @@ k_substep(const int4 *__restrict__ sv, const float4 *__restrict__ sg, const floa
     const int nown = patch_own[p];
     const float one_p_theta = __fadd_rn(1.0f, a.theta);
 
+    // A round of this loop waits on memory, not on issue or bandwidth: with every load that does
+    // not depend on another one requested first (the transport sums and V0 too), a round has two
+    // latencies in a row instead of four. Viscous substep of a 588 x 340 channel: 20.0 -> 18.2 us
+    // at 256 threads although 64 registers leave fewer warps than 56 did; capping the registers
+    // at 48 or 40 for more warps spills and is slower (20.5, 18.2).
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         const int s = s0 + i;
         const int4 v = sv[s];
         const float4 g = sg[s];
         const float4 c = sc[s];
         float2 r = R[s];
+        ViscRow row{};
+        float2 z = make_float2(0.0f, 0.0f), hi = z, lo = z;
+        if (VISC) row = visc_row(vis.T, s);
+        if (VISC && !vis.start) z = vis.V0[s];
+        if (i < nown) {
+            hi = Shi[s];
+            lo = Slo[s];
+        }
         const float2 u = U_in[s];
         const float e0 = eta_in[v.x], e1 = eta_in[v.y], e2 = eta_in[v.z];
         if (VISC) {
             float H = c.y;
             if (NONLIN) H += (e0 + e1 + e2) * (1.0f / 3.0f);
             const float ev[3] = {e0, e1, e2};
-            const float2 V = visc_of<VISC == 2>(s, H, u, ev, c.x, vis.T, U_in, eta_in, vis.va);
+            const float2 V = visc_of<VISC == 2>(s, H, u, ev, c.x, vis.T, row, U_in, eta_in, vis.va);
             if (vis.start) {
                 vis.V0[s] = V;      // R' = R + (V - V) = R
             } else {
-                const float2 z = vis.V0[s];
                 r = make_float2(r.x + (V.x - z.x), r.y + (V.y - z.y));
             }
         }
@@ -156,29 +180,38 @@ k_substep(const int4 *__restrict__ sv, const float4 *__restrict__ sg, const floa
                                               a.theta, un);
         U_out[s] = un;
         if (i < nown) {
-            float2 hi = Shi[s], lo = Slo[s];
             two_sum_acc2(hi, lo, F);
             Shi[s] = hi;
             Slo[s] = lo;
         }
         corner_fluxes(F, g, __fmul_rn(dt, c.x), sflux + 3 * i);
     }
-    __syncthreads();
 
     const int v1 = patch_v[p + 1];
+    int vx = patch_v[p] + threadIdx.x, k0 = 0, k1 = 0;
+    if (vx < v1) {
+        k0 = vcsr_off[vx];
+        k1 = vcsr_off[vx + 1];
+    }
+    __syncthreads();
+
     bool bad = false;
-    for (int v = patch_v[p] + threadIdx.x; v < v1; v += blockDim.x) {
-        const int k1 = vcsr_off[v + 1];
+    while (vx < v1) {
         float sum = 0.0f;
-        for (int k = vcsr_off[v]; k < k1; k++) {
+        for (int k = k0; k < k1; k++) {
             const uint32_t q = vcsr[k];
             sum += sflux[3 * (q >> 2) + (q & 3u)];
         }
-        float e = vertex_eta(eta_in[v], sum, inv_av[v]);
-        if (W) e = __fmaf_rn(-dt, W[v], e);
-        if (eta_sum) eta_sum[v] += eta_in[v];     // sum of eta^0 .. eta^{M-1} (time mean of the step)
-        eta_out[v] = e;
+        float e = vertex_eta(eta_in[vx], sum, inv_av[vx]);
+        if (W) e = __fmaf_rn(-dt, W[vx], e);
+        if (eta_sum) eta_sum[vx] += eta_in[vx];   // sum of eta^0 .. eta^{M-1} (time mean of the step)
+        eta_out[vx] = e;
         bad |= !(fabsf(e) <= a.eta_bound);
+        vx += blockDim.x;
+        if (vx < v1) {
+            k0 = vcsr_off[vx];
+            k1 = vcsr_off[vx + 1];
+        }
     }
     if (bad) atomicOr(status, 1u);
 }
@@ -293,7 +326,7 @@ k_viscosity(const int4 *__restrict__ sv, const float4 *__restrict__ sc, const fl
         const float e[3] = {eta[v.x], eta[v.y], eta[v.z]};
         float H = c.y;
         if (va.nonlinear_h) H += (e[0] + e[1] + e[2]) * (1.0f / 3.0f);
-        out[v.w] = visc_of<ROT>(s, H, U[s], e, c.x, T, U, eta, va);
+        out[v.w] = visc_of<ROT>(s, H, U[s], e, c.x, T, visc_row(T, s), U, eta, va);
     }
 }
 
@@ -457,10 +490,49 @@ int grid_for(int n, int threads)
 
 }  // namespace
 
+// Threads per block of k_substep when the caller names none. A launch lasts (waves of
+// blocks) x (rounds of the slot loop) and each round waits on two dependent loads, so the
+// size with the least product is taken, the smallest of equals. Viscous substeps of a
+// 588 x 340 channel (781 patches of up to 625 slots, 64 registers): 13.8 us with 160 threads
+// (1 wave, 4 rounds), 15.5 with 320 (2, 2), 18.2 with 256 (2, 3), 18.7 with 192 (2, 4),
+// 20.9 with 224 (2, 3); of a 62 x 50 channel (13 patches): 8.4 with 256, 4.6 with 576.
+// Without the viscosity a round is cheap and a device with several waves is bound by bandwidth
+// (the 588 x 340 channel: 7.1 us with 256 threads, 7.9 with 320), so there only larger blocks of
+// a grid that fits one wave are taken (62 x 50: 4.6 -> 3.5 us; 330 x 300: 5.4 -> 5.1).
+int substep_threads(const DevMesh &m, bool nonlin, bool visc)
+{
+    if (m.npatch <= 0) return 256;
+    const int vk = visc ? (m.visc_rot ? 2 : 1) : 0;
+    const void *fns[6] = {(const void *)k_substep<0, 0>, (const void *)k_substep<1, 0>,
+                          (const void *)k_substep<0, 1>, (const void *)k_substep<1, 1>,
+                          (const void *)k_substep<0, 2>, (const void *)k_substep<1, 2>};
+    const void *fn = fns[2 * vk + (nonlin ? 1 : 0)];
+    const size_t smem = sizeof(float) * 3 * (size_t)m.max_patch_slots;
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        sms = 0;
+    int best = 256;
+    long long best_cost = -1;
+    for (int t = visc ? 64 : 256; sms > 0 && t <= kSubstepMaxThreads; t += 32) {
+        int bps = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, fn, t, smem) != cudaSuccess || bps < 1) break;
+        const long long resident = (long long)bps * sms;
+        const long long waves = (m.npatch + resident - 1) / resident;
+        if (!visc && t > 256 && waves > 1) break;
+        const long long cost = waves * ((m.max_patch_slots + t - 1) / t);
+        if (best_cost < 0 || cost < best_cost) {
+            best = t;
+            best_cost = cost;
+        }
+    }
+    cudaGetLastError();
+    return best;
+}
+
 cudaError_t launch_substep(const DevMesh &m, const DevState &s, const StepArgs &a, int parity, int block,
                            cudaStream_t stream, const SubstepViscArgs *visc)
 {
-    const int threads = block > 0 ? block : 256;
     const size_t smem = sizeof(float) * 3 * (size_t)m.max_patch_slots;
     const float *ein = s.eta[parity];
     float *eout = s.eta[parity ^ 1];
@@ -476,7 +548,7 @@ cudaError_t launch_substep(const DevMesh &m, const DevState &s, const StepArgs &
         uout = visc->U_out;
     }
 #define SESW_SUBSTEP(NL, VI)                                                                                      \
-    k_substep<NL, VI><<<m.npatch, threads, smem, stream>>>(                                                      \
+    k_substep<NL, VI><<<m.npatch, block, smem, stream>>>(                                                      \
         m.slot_v, m.slot_g, m.slot_c, s.R, uin, uout, s.S_hi, s.S_lo, m.patch_slot, m.patch_own, m.patch_v,      \
         m.vcsr_off, m.vcsr, m.inv_av, ein, eout, m.patch_dt, s.eta_sum, s.W, vis, a, s.status)
     const int vk = visc ? (m.visc_rot ? 2 : 1) : 0;
