@@ -608,6 +608,8 @@ int build_halos(HostMesh &hm, std::string &err)
     hm.max_patch_halo = 0;
     hm.max_patch_csr = 0;
     std::vector<int> halo;
+    // patch that last listed a vertex as halo, and the vertex's place there
+    std::vector<int> seen(hm.patch_v[np], -1), place(hm.patch_v[np], 0);
     for (int p = 0; p < np; p++) {
         const int vlo = hm.patch_v[p], vhi = hm.patch_v[p + 1], nown = vhi - vlo;
         halo.clear();
@@ -615,10 +617,13 @@ int build_halos(HostMesh &hm, std::string &err)
             const int4 c = hm.slot_v[s];
             const int cv[3] = {c.x, c.y, c.z};
             for (int k = 0; k < 3; k++)
-                if (cv[k] < vlo || cv[k] >= vhi) halo.push_back(cv[k]);
+                if ((cv[k] < vlo || cv[k] >= vhi) && seen[cv[k]] != p) {
+                    seen[cv[k]] = p;
+                    halo.push_back(cv[k]);
+                }
         }
         std::sort(halo.begin(), halo.end());
-        halo.erase(std::unique(halo.begin(), halo.end()), halo.end());
+        for (size_t j = 0; j < halo.size(); j++) place[halo[j]] = nown + (int)j;
         const int nloc = nown + (int)halo.size();
         if (nloc > 65535) {
             err = "a patch has more than 65535 local vertices; the persistent kernel needs smaller patches";
@@ -632,7 +637,7 @@ int build_halos(HostMesh &hm, std::string &err)
                 if (cv[k] >= vlo && cv[k] < vhi)
                     l[k] = (unsigned short)(cv[k] - vlo);
                 else
-                    l[k] = (unsigned short)(nown + (std::lower_bound(halo.begin(), halo.end(), cv[k]) - halo.begin()));
+                    l[k] = (unsigned short)place[cv[k]];
             }
             hm.slot_l[s] = make_ushort4(l[0], l[1], l[2], 0);
         }
