@@ -811,6 +811,7 @@ static int upload_batch(sesw_ctx *c, const sesw_mesh *meshes, int n)
         d.max_patch_csr = hm.max_patch_csr;
     }
 
+    if (!c->host_words) CK(c, cudaMallocHost(&c->host_words, kHostWords * sizeof(double)));
     sesw::DevState &s = c->ds;
     TRY(zalloc(c, &s.eta[0], hm.nv, "eta"));
     TRY(zalloc(c, &s.eta[1], hm.nv, "eta"));
@@ -1290,10 +1291,10 @@ int sesw_get_state(sesw_ctx *c, double *eta, double *U, double *Umean, int where
     if (eta) CK(c, cudaMemcpyAsync(eta, se, sizeof(double) * nv, cudaMemcpyDeviceToHost, c->stream));
     if (U) CK(c, cudaMemcpyAsync(U, su, sizeof(double) * 2 * ne, cudaMemcpyDeviceToHost, c->stream));
     if (Umean) CK(c, cudaMemcpyAsync(Umean, sm, sizeof(double) * 2 * ne, cudaMemcpyDeviceToHost, c->stream));
-    unsigned status = 0;
-    CK(c, cudaMemcpyAsync(&status, c->ds.status, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
+    unsigned *status = (unsigned *)c->host_words;
+    CK(c, cudaMemcpyAsync(status, c->ds.status, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
     CK(c, cudaStreamSynchronize(c->stream));
-    if (status & 1u) return fail(c, SESW_EUNSTABLE, "non-finite or out-of-bound elevation detected");
+    if (*status & 1u) return fail(c, SESW_EUNSTABLE, "non-finite or out-of-bound elevation detected");
     return SESW_OK;
 }
 
@@ -1303,8 +1304,8 @@ int sesw_diagnostics(sesw_ctx *c, double *volume, double *energy)
     if (!c->have_mesh || !c->have_params) return fail(c, SESW_ESTATE, "mesh and parameters must be set before diagnostics");
     DeviceGuard dg(c->device);
     CK(c, sesw::launch_diagnostics(c->dm, c->ds, c->args, c->parity, c->diag_blocks, c->stream));
-    double out[2] = {0.0, 0.0};
-    CK(c, cudaMemcpyAsync(out, c->ds.diag_out, sizeof out, cudaMemcpyDeviceToHost, c->stream));
+    const double *out = c->host_words;
+    CK(c, cudaMemcpyAsync(c->host_words, c->ds.diag_out, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     CK(c, cudaStreamSynchronize(c->stream));
     if (volume) *volume = out[0];
     if (energy) *energy = out[1];
@@ -1470,6 +1471,7 @@ void sesw_destroy(sesw_ctx *c)
             for (cudaEvent_t ev : {c->in_done[b], c->in_free[b], c->out_ready[b], c->out_done[b]})
                 if (ev) cudaEventDestroy(ev);
         if (c->status_h) cudaFreeHost(c->status_h);
+        if (c->host_words) cudaFreeHost(c->host_words);
         cudaGetLastError();
     }
     delete c;

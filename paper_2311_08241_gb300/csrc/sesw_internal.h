@@ -379,6 +379,8 @@ cudaError_t launch_bwd_layer_tc(const BwdLayerArgs &b, unsigned *status, cudaStr
 }  // namespace sesw
 
 // The context behind the C-ABI handle.
+constexpr int kHostWords = 2048;   // doubles in sesw_ctx::host_words
+
 struct sesw_ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
@@ -428,6 +430,10 @@ struct sesw_ctx {
     cudaEvent_t in_done[2] = {}, in_free[2] = {}, out_ready[2] = {}, out_done[2] = {};
     double *stage_in[2] = {nullptr, nullptr};    // [2 ne] forcing in transit
     double *stage_out[2] = {nullptr, nullptr};   // [nv + 4 ne] state in transit
+    // pinned, kHostWords doubles: where the small results of blocking calls land (the status word,
+    // the diagnostics, the surrogate's loss and residual sums). A copy to pageable memory is staged
+    // by the driver and waited for one by one. Allocated with the context's first mesh.
+    double *host_words = nullptr;
     unsigned *status_h = nullptr;                // [2] pinned: the status word as of each buffer's last download
     int in_idx = 0, out_idx = 0;
     uint64_t out_seq = 0;

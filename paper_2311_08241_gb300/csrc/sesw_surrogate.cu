@@ -518,6 +518,16 @@ __global__ void k_apply_elems(int E, int nslot, const int4 *__restrict__ sv, con
     }
 }
 
+// Every slot's transport back from the per-element copy taken before k_apply_elems.
+__global__ void k_restore_elems(int nslot, const int4 *__restrict__ sv, const float *__restrict__ U0e,
+                                float2 *__restrict__ Us)
+{
+    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < nslot; s += gridDim.x * blockDim.x) {
+        const int w = sv[s].w, e = w >= 0 ? w : -1 - w;
+        Us[s] = make_float2(U0e[2 * e], U0e[2 * e + 1]);
+    }
+}
+
 // eta^{n+1} = eta^n - tau div <<U>> (median-dual divergence, as the plain vertex pass)
 // and eta_bar = eta^n + s_oeta o_v.
 __global__ void k_apply_verts(int V, const int *__restrict__ voff, const int *__restrict__ vinc,
@@ -642,8 +652,6 @@ struct Surrogate {
     float *d_eta = nullptr, *d_U = nullptr, *d_R = nullptr, *d_te = nullptr, *d_tv = nullptr;
     // inference
     float *cur_eta = nullptr, *cur_U = nullptr, *cur_R = nullptr, *etabar = nullptr;
-    float *save_eta = nullptr;
-    float2 *save_U = nullptr;
     double *stage = nullptr;    // host samples in transit: 2 V + 8 E doubles
     unsigned *status = nullptr; // the context's device status word (timeout bit of the tensor-core waits)
 };
@@ -984,8 +992,6 @@ int sesw_surrogate_init(sesw_ctx *c, int32_t capacity, int32_t seed)
     STRY(sesw::salloc(c, &S.cur_U, 2 * (size_t)E));
     STRY(sesw::salloc(c, &S.cur_R, 2 * (size_t)E));
     STRY(sesw::salloc(c, &S.etabar, (size_t)V));
-    STRY(sesw::salloc(c, &S.save_eta, (size_t)V));
-    STRY(sesw::salloc(c, &S.save_U, (size_t)c->dm.nslot));
     STRY(sesw::salloc(c, &S.stage, 2 * (size_t)V + 8 * (size_t)E));
     SCK(cudaStreamSynchronize(c->stream));
     return SESW_OK;
@@ -1135,7 +1141,7 @@ int sesw_surrogate_fit_scales(sesw_ctx *c, int64_t nsamples, double length_scale
     return sesw_surrogate_scales(c, nullptr, sc);
 }
 
-static int run_sample(sesw_ctx *c, long i, bool grad, bool adam, double *loss)
+static int run_sample(sesw_ctx *c, long i, bool grad, bool adam, double *loss, float *grad_out = nullptr)
 {
     Surrogate &S = *c->sur;
     sesw::features_of(S, c, i);
@@ -1154,11 +1160,12 @@ static int run_sample(sesw_ctx *c, long i, bool grad, bool adam, double *loss)
             SCK(sesw::pack_tc(S, c->stream));
         }
     }
-    if (loss) {
-        double l = 0.0;
-        SCK(cudaMemcpyAsync(&l, S.red, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+    if (loss || grad_out) {
+        if (loss) SCK(cudaMemcpyAsync(c->host_words, S.red, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+        if (grad_out)
+            SCK(cudaMemcpyAsync(grad_out, S.grad, sizeof(float) * S.nparam, cudaMemcpyDeviceToHost, c->stream));
         SCK(cudaStreamSynchronize(c->stream));
-        *loss = l;
+        if (loss) *loss = c->host_words[0];
     }
     return SESW_OK;
 }
@@ -1202,12 +1209,7 @@ int sesw_surrogate_gradient(sesw_ctx *c, int64_t index, float *grad, double *los
     STRY(need_sur(c));
     Surrogate &S = *c->sur;
     if (index < 0 || index >= S.cap) return sesw::ctx_fail(c, SESW_EINVAL, "sample index out of range");
-    STRY(run_sample(c, index, true, false, loss));
-    if (grad) {
-        SCK(cudaMemcpyAsync(grad, S.grad, sizeof(float) * S.nparam, cudaMemcpyDeviceToHost, c->stream));
-        SCK(cudaStreamSynchronize(c->stream));
-    }
-    return SESW_OK;
+    return run_sample(c, index, true, false, loss, grad);
 }
 
 int sesw_surrogate_predict(sesw_ctx *c, int64_t index, double *out_e, double *out_v)
@@ -1244,11 +1246,10 @@ int sesw_surrogate_advance(sesw_ctx *c, int32_t nsteps, double resid_tol, int32_
     const int nb = 152 * 4;
     for (int n = 0; n < nsteps; n++) {
         float *eta0 = c->ds.eta[c->parity];
-        // the current state as network input, and a copy for the fallback
+        // the current state as network input; it is also what the fallback starts from (eta0 is only
+        // read below, and every copy of an element holds its owner's transport, cur_U)
         sesw::k_take_state<<<sesw::grid1(std::max(S.V, S.E)), 256, 0, c->stream>>>(
             S.V, S.E, eta0, c->ds.U, c->ds.R, S.eslot, S.cur_eta, S.cur_U, S.cur_R);
-        SCK(cudaMemcpyAsync(S.save_eta, eta0, sizeof(float) * S.V, cudaMemcpyDeviceToDevice, c->stream));
-        SCK(cudaMemcpyAsync(S.save_U, c->ds.U, sizeof(float2) * c->dm.nslot, cudaMemcpyDeviceToDevice, c->stream));
         sesw::k_features<<<sesw::grid1(std::max(S.V, S.E)), 256, 0, c->stream>>>(
             S.V, S.E, S.cur_eta, S.cur_U, S.cur_R, c->dm.h0_v, S.eH0, S.ef, S.scales, S.xv, S.xe);
         SCK(sesw::forward(S, c->stream, false));
@@ -1263,8 +1264,8 @@ int sesw_surrogate_advance(sesw_ctx *c, int32_t nsteps, double resid_tol, int32_
                                                     c->args.theta, (float)c->params.M, c->params.nonlinear_h,
                                                     S.red + 16);
         SCK(cudaGetLastError());
-        std::vector<double> h(2 * nb);
-        SCK(cudaMemcpyAsync(h.data(), S.red + 16, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, c->stream));
+        const double *h = c->host_words;
+        SCK(cudaMemcpyAsync(c->host_words, S.red + 16, sizeof(double) * 2 * nb, cudaMemcpyDeviceToHost, c->stream));
         SCK(cudaStreamSynchronize(c->stream));
         double a = 0.0, b = 0.0;
         for (int k = 0; k < nb; k++) {
@@ -1276,8 +1277,9 @@ int sesw_surrogate_advance(sesw_ctx *c, int32_t nsteps, double resid_tol, int32_
             c->parity ^= 1;
         } else {
             // the plain subcycle takes this step instead
-            SCK(cudaMemcpyAsync(eta0, S.save_eta, sizeof(float) * S.V, cudaMemcpyDeviceToDevice, c->stream));
-            SCK(cudaMemcpyAsync(c->ds.U, S.save_U, sizeof(float2) * c->dm.nslot, cudaMemcpyDeviceToDevice, c->stream));
+            sesw::k_restore_elems<<<sesw::grid1(c->dm.nslot), 256, 0, c->stream>>>(c->dm.nslot, c->dm.slot_v, S.cur_U,
+                                                                                   c->ds.U);
+            SCK(cudaGetLastError());
             STRY(sesw::ctx_enqueue_step(c));
             fb++;
         }
