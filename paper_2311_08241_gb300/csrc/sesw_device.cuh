@@ -12,7 +12,6 @@ namespace sesw {
 // substep (gradients, transports, sums) are (x, y) pairs, so they take half the instructions.
 __device__ __forceinline__ float2 pair(float a, float b) { return make_float2(a, b); }
 __device__ __forceinline__ float2 splat(float a) { return make_float2(a, a); }
-__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
 
 // Error-free accumulation of x into the pair (hi, lo): after the call hi + lo equals
 // the old hi + lo + x up to the rounding of lo (Knuth's two-sum). The explicit

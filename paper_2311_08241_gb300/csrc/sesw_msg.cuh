@@ -9,9 +9,6 @@
 
 namespace sesw {
 
-// x rounded to the nearest bfloat16 value
-__device__ __forceinline__ float bf16_value(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
-
 // Element message of one hidden channel: L (sum_k dphi_k/dx h_k, sum_k dphi_k/dy h_k) over the
 // corners, g = (dphi0/dx, dphi0/dy, dphi1/dx, dphi1/dy) and dphi_2 = -(dphi_0 + dphi_1).
 __device__ __forceinline__ float2 msg_elem_grad(float4 g, float h0, float h1, float h2, float L)

@@ -356,7 +356,6 @@ struct TmemSlots {
 // at P.off_flux.
 template <int SPT>
 struct GlobalSlots {
-    static constexpr int kWords = 0;
     static constexpr bool kTmem = false;
     static constexpr bool kFluxShared = false;
     __device__ static __forceinline__ void store(uint32_t, int, const SlotData &) {}
@@ -476,17 +475,15 @@ struct SmemLayout {
     int off_flux, off_g, off_c, off_r, off_l, off_off, off_csr, off_inv, off_halo;
     int inc8, zero_off;
     size_t total_plain;     // elevation, corner fluxes and the zero word
-    size_t total_vcached;   // ... and the vertices' data: 1/A_v, halo ids, incidences
-    size_t total_cached;    // ... and the slots' static data
+    size_t total_cached;    // ... the vertices' data (1/A_v, halo ids, incidences) and the slots' static data
 };
 
 inline size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
 
 // Shared-memory layout of a patch: [elevation of own and halo vertices | corner fluxes, zero
 // word | 1/A_v, halo ids, incidences | per slot: gradients, coefficients, forcing, corners].
-// The kernels that keep everything on chip use the whole layout (CACHED = 1), those for larger
-// patches the part up to the incidences (CACHED = 2: the slots' static data then come from L2),
-// the streaming kernels only the first part.
+// The SESM kernel that keeps everything on chip uses the whole layout, the streaming kernels only
+// the first part (the kernels with tensor memory have their own, se_layout and sesm_layout).
 inline SmemLayout smem_layout(const PatchMax &m)
 {
     SmemLayout L;
@@ -510,7 +507,6 @@ inline SmemLayout smem_layout(const PatchMax &m)
     L.inc8 = m.deg > kIncWidth ? 0 : (L.zero_off + 4 <= 65535 ? 1 : (L.zero_off / 4 + 1 <= 65535 ? 2 : 0));
     const size_t inc_end = o + sizeof(unsigned short) * kIncWidth * (size_t)m.vertices;
     o = L.inc8 ? align16(inc_end) : csr_end;
-    L.total_vcached = o;
     L.off_g = (int)o;
     o += sizeof(float4) * (size_t)m.slots;
     L.off_c = (int)o;
