@@ -60,7 +60,7 @@ def parse(argv=None):
                     help="freshwater flux W of Eq. (4.5): seeded random field of this amplitude (m/s)")
     ap.add_argument("--patch-vertices", type=int, default=None,
                     help="graph-mode patch size (default 256; with --visc, one wave of the fused kernel)")
-    ap.add_argument("--block-threads", type=int, default=256)
+    ap.add_argument("--block-threads", type=int, default=None)
     ap.add_argument("--blocks-per-sm", type=int, default=0)
     ap.add_argument("--e2e-steps", type=int, default=400)
     ap.add_argument("--cpu-seconds", type=float, default=10.0)
@@ -789,7 +789,8 @@ def run_ours(args, world, rank, local):
         else:
             pv = 256
     sim.sesw_set_patch_vertices(pv)
-    sim.sesw_set_block_threads(args.block_threads)
+    if args.block_threads:
+        sim.sesw_set_block_threads(args.block_threads)
     sim.sesw_set_blocks_per_sm(args.blocks_per_sm)
     sim.sesw_mesh_upload(case.mesh)
     sim.sesw_set_params(case.params)

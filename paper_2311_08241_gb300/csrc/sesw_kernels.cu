@@ -497,12 +497,14 @@ int grid_for(int n, int threads)
 
 }  // namespace
 
-// Threads per block of k_substep when the caller names none. A launch lasts (waves of
-// blocks) x (rounds of the slot loop) and each round waits on two dependent loads, so the
-// size with the least product is taken, the smallest of equals. Viscous substeps of a
-// 588 x 340 channel (781 patches of up to 625 slots, 64 registers): 13.8 us with 160 threads
-// (1 wave, 4 rounds), 15.5 with 320 (2, 2), 18.2 with 256 (2, 3), 18.7 with 192 (2, 4),
-// 20.9 with 224 (2, 3); of a 62 x 50 channel (13 patches): 8.4 with 256, 4.6 with 576.
+// Threads per block of k_substep when the caller names none. A launch lasts (waves of blocks) x
+// (rounds of the slot loop) and each round waits on two dependent loads, so the size with the
+// least product is taken, the smallest of equals; the rounds of a mean patch and of the largest
+// one count alike. Viscous substeps of a 588 x 340 channel (781 patches of 595 slots on average,
+// 625 at most, 64 registers): 13.8 us with 160 threads (1 wave, 4 rounds), 15.5 with 320 (2, 2),
+// 18.2 with 256 (2, 3), 18.7 with 192 (2, 4), 20.9 with 224 (2, 3); with 608 patches of 753 slots
+// on average, 13.1 us with 256 (1 wave, 3 rounds) and 14.3 with 224 (1, 4); of a 62 x 50 channel
+// (13 patches), 8.4 us with 256 and 4.6 with 576.
 // Without the viscosity a round is cheap and a device with several waves is bound by bandwidth
 // (the 588 x 340 channel: 7.1 us with 256 threads, 7.9 with 320), so there only larger blocks of
 // a grid that fits one wave are taken (62 x 50: 4.6 -> 3.5 us; 330 x 300: 5.4 -> 5.1).
@@ -519,6 +521,7 @@ int substep_threads(const DevMesh &m, bool nonlin, bool visc)
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         sms = 0;
+    const int mean = (m.nslot + m.npatch - 1) / m.npatch;
     int best = 256;
     long long best_cost = -1;
     for (int t = visc ? 64 : 256; sms > 0 && t <= kSubstepMaxThreads; t += 32) {
@@ -527,7 +530,7 @@ int substep_threads(const DevMesh &m, bool nonlin, bool visc)
         const long long resident = (long long)bps * sms;
         const long long waves = (m.npatch + resident - 1) / resident;
         if (!visc && t > 256 && waves > 1) break;
-        const long long cost = waves * ((m.max_patch_slots + t - 1) / t);
+        const long long cost = waves * ((mean + t - 1) / t + (m.max_patch_slots + t - 1) / t);
         if (best_cost < 0 || cost < best_cost) {
             best = t;
             best_cost = cost;
