@@ -123,14 +123,20 @@ int graph_threads(const sesw_ctx *c)
     return sesw::substep_threads(c->dm, c->params.nonlinear_h != 0, c->visc_on);
 }
 
+// Clears the step-mean elevation's sum at the start of a step whose kernels do not start it themselves: the
+// persistent SE kernels do, graph mode only adds to it, and the SESM kernels leave it alone (enabled under
+// SE, it then reads zero).
+cudaError_t clear_eta_sum(const sesw_ctx *c, cudaStream_t stream)
+{
+    if (!c->ds.eta_sum || (c->mode == SESW_MODE_PERSISTENT && c->params.scheme == 0)) return cudaSuccess;
+    return cudaMemsetAsync(c->ds.eta_sum, 0, sizeof(float) * (size_t)c->dm.nv, stream);
+}
+
 int capture_step_graph(sesw_ctx *c, int parity, cudaGraphExec_t *out)
 {
     cudaGraph_t g = nullptr;
     CK(c, cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
-    cudaError_t e = cudaSuccess;
-    // (the persistent kernels start the sum themselves)
-    if (c->ds.eta_sum && c->mode != SESW_MODE_PERSISTENT)
-        e = cudaMemsetAsync(c->ds.eta_sum, 0, sizeof(float) * (size_t)c->dm.nv, c->cap_stream);
+    cudaError_t e = clear_eta_sum(c, c->cap_stream);
     if (e != cudaSuccess) {
     } else if (c->mode == SESW_MODE_PERSISTENT) {
         e = c->params.scheme == 1
@@ -211,6 +217,7 @@ int capture_step_graph(sesw_ctx *c, int parity, cudaGraphExec_t *out)
 int enqueue_step(sesw_ctx *c)
 {
     if (c->mode == SESW_MODE_PERSISTENT && !c->persist_graph_ok) {
+        CK(c, clear_eta_sum(c, c->stream));
         if (c->params.scheme == 1)
             CK(c, sesw::launch_persistent_sesm(c->dm, c->ds, c->args, c->params.M, c->parity, 1, c->packs, c->stream));
         else
@@ -1261,6 +1268,7 @@ int sesw_advance(sesw_ctx *c, int32_t nsteps)
     for (int n = 0; n < nsteps;) {
         const int k = steps_per_launch(c, nsteps - n);
         if (k > 1) {
+            CK(c, clear_eta_sum(c, c->stream));
             if (c->params.scheme == 1)
                 CK(c, sesw::launch_persistent_sesm(c->dm, c->ds, c->args, c->params.M, c->parity, k, c->packs, c->stream));
             else
