@@ -83,7 +83,6 @@ __device__ __forceinline__ void persistent_patch(const PArgs &P, const int p, co
     float *s_inv = reinterpret_cast<float *>(smem_raw + P.off_inv);
     int *s_halo = reinterpret_cast<int *>(smem_raw + P.off_halo);
     const uint32_t slo_at = team + (uint32_t)P.off_slo;
-    float2 *s_slo = reinterpret_cast<float2 *>(smem_raw + P.off_slo);
 
     for (int i = tid; i < nown; i += T) seta[i] = P.eta_in[v0 + i];
     for (int i = tid; i < nhalo; i += T) seta[nown + i] = P.eta_in[P.halo_v[hb + i]];
@@ -127,7 +126,7 @@ __device__ __forceinline__ void persistent_patch(const PArgs &P, const int p, co
         u[j] = in ? P.U[s] : make_float2(0.0f, 0.0f);
         shi[j] = make_float2(0.0f, 0.0f);
         if (!kSloShared) slo[j] = make_float2(0.0f, 0.0f);
-        if (kSloShared && i < nsp) s_slo[i] = make_float2(0.0f, 0.0f);
+        if (kSloShared && i < nsp) sts2(slo_at + 8 * i, make_float2(0.0f, 0.0f));
     }
     if (TS::kTmem) tmem_wait_st();
     team_sync(bar, T);
@@ -225,14 +224,15 @@ __device__ __forceinline__ void persistent_patch(const PArgs &P, const int p, co
         team_sync(bar, T);
         if (!more) break;
         if (++ms == P.M) {
-            // a step ends: the sums of the next one start from zero
+            // a step ends: the sums of the next one start from zero (the low parts in shared memory by
+            // sts2, which keeps its order to the lds2 of the next substep: no barrier lies between)
             ms = 0;
 #pragma unroll
             for (int j = 0; j < SPT; j++) {
                 const int i = tid + j * T;
                 shi[j] = make_float2(0.0f, 0.0f);
                 if (!kSloShared) slo[j] = make_float2(0.0f, 0.0f);
-                if (kSloShared && i < nsp) s_slo[i] = make_float2(0.0f, 0.0f);
+                if (kSloShared && i < nsp) sts2(slo_at + 8 * i, make_float2(0.0f, 0.0f));
             }
         }
     }
@@ -246,7 +246,7 @@ __device__ __forceinline__ void persistent_patch(const PArgs &P, const int p, co
             P.U[s0 + i] = u[j];
             if (i < nown_s) {
                 const int w = P.sv[s0 + i].w;
-                const float2 lo = kSloShared ? s_slo[i] : slo[kSloShared ? 0 : j];
+                const float2 lo = kSloShared ? lds2(slo_at + 8 * i) : slo[kSloShared ? 0 : j];
                 P.Umean[w] = make_float2((shi[j].x + lo.x) * a.inv_M, (shi[j].y + lo.y) * a.inv_M);
             }
         }
