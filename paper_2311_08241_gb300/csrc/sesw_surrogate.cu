@@ -974,7 +974,7 @@ int sesw_surrogate_init(sesw_ctx *c, int32_t capacity, int32_t seed)
     size_t part_len = 0;
     for (size_t l = 0; l < S.L.size(); l++) {
         const int n = l % 2 == 0 ? (l == 0 ? V : E) : (l == 1 ? E : V);   // rows of layer l (see S.L)
-        const int nb = S.L[l].tc >= 0 ? sesw::bwd_layer_ctas(n)
+        const int nb = S.L[l].tc >= 0 ? sesw::bwd_layer_parts(n)
                                       : (n + sesw::small_rows(n) - 1) / sesw::small_rows(n);
         S.part_off.push_back(part_len);
         S.part_nb.push_back(nb);

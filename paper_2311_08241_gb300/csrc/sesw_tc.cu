@@ -30,7 +30,7 @@ namespace sesw {
 
 namespace {
 
-constexpr int TC_M = 128;        // rows per CTA: one MMA with M = 128
+constexpr int TC_M = kMsgTile;   // rows per tile: one MMA with M = 128
 constexpr int TC_N = 64;         // output columns: the hidden width
 constexpr int TC_THREADS = 256;  // eight warps: warp w reads TMEM lanes 32 (w % 4) .. + 31, columns 32 (w / 4) .. + 31
 
@@ -442,7 +442,7 @@ k_msg_layer_tc(const MsgLayerArgs a, const uint4 *__restrict__ Wp, const float *
 //   dh    = dh_in + the gradient that the layers behind sent through their messages (gathered
 //           here from g0, g1, where they are per row of the other kind)
 //   dA    = dh (1 - Y^2)                                         (FP32)
-//   G     = Z^T dA, column sums of dA: weight and bias gradient  (partial per CTA)
+//   G     = Z^T dA, column sums of dA: weight and bias gradient  (partial sums, see bwd_layer_part)
 //   dZ    = dA W^T; dh_out = dh + dZ[:, 0:64]; m0, m1 = the other 64-wide blocks of dZ, the
 //           gradients of the layer's messages
 // dA is not a bfloat16 value, so each of its elements is split into two bfloat16 parts,
@@ -502,6 +502,47 @@ k_bwd_layer_tc(const BwdLayerArgs b, unsigned *__restrict__ status, long long wa
     float bsum[8];
 #pragma unroll
     for (int t = 0; t < 8; t++) bsum[t] = 0.0f;
+    // The CTA's sums so far (G in tensor memory, bias in registers) to a partial sum; zeros after a wait that
+    // gave up. The bias adds the 32 threads of a channel octet in a fixed order.
+    auto flush = [&](int part) {
+        {
+            const int t0 = tid >> 3;
+#pragma unroll
+            for (int t = 0; t < 8; t++) {
+                s_bias[t0 * TC_N + c8 + t] = bsum[t];
+                bsum[t] = 0.0f;
+            }
+        }
+        __syncthreads();
+        float *out = b.partial + (size_t)part * ((size_t)K * TC_N + TC_N);
+        if (tid < TC_N) {
+            float x = 0.0f;
+            for (int k = 0; k < 32; k++) x += s_bias[k * TC_N + tid];
+            out[(size_t)K * TC_N + tid] = x;
+        }
+        // G rows i: features 0..127 from the first accumulator, 128..191 from the second's lanes 64..127
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        const int quarter = warp & 3, half = warp >> 2;
+#pragma unroll
+        for (int mt = 0; mt < (KIND == 0 ? 2 : 1); mt++) {
+            const int i = mt * 64 + quarter * 32 + lane;
+#pragma unroll
+            for (int q = 2 * half; q < 2 * half + 2; q++) {
+                float v[16];
+                if (s_ok) {
+                    tmem_ld16(tmem_base + ((uint32_t)(quarter * 32) << 16) + 128 + 64 * mt + q * 16, v);
+                } else {
+#pragma unroll
+                    for (int t = 0; t < 16; t++) v[t] = 0.0f;
+                }
+                if (mt == 0 || quarter >= 2) {
+                    float4 *dst = reinterpret_cast<float4 *>(out + (size_t)i * TC_N + q * 16);
+#pragma unroll
+                    for (int t = 0; t < 16; t += 4) dst[t / 4] = make_float4(v[t], v[t + 1], v[t + 2], v[t + 3]);
+                }
+            }
+        }
+    };
     uint32_t parity = 0;
     int done = 0;
     for (int tile = blockIdx.x; tile < ntile; tile += gridDim.x, parity ^= 1u, done++) {
@@ -622,7 +663,7 @@ k_bwd_layer_tc(const BwdLayerArgs b, unsigned *__restrict__ status, long long wa
 #pragma unroll
                 for (int mt = 0; mt < (KIND == 0 ? 2 : 1); mt++) {
                     const uint64_t ad = umma_desc_sw(z0 + mt * TILE_BLOCK + ks * 2048, TILE_BLOCK, 1024);
-                    mma_bf16(tmem + 128 + 64 * mt, ad, bh, id2, done > 0 || ks > 0);
+                    mma_bf16(tmem + 128 + 64 * mt, ad, bh, id2, done % kGradTiles > 0 || ks > 0);
                     mma_bf16(tmem + 128 + 64 * mt, ad, bl, id2, 1);
                 }
             }
@@ -673,51 +714,22 @@ k_bwd_layer_tc(const BwdLayerArgs b, unsigned *__restrict__ status, long long wa
             __syncthreads();
             put(b.m1, false);
         }
+        if ((done + 1) % kGradTiles == 0 || tile + (int)gridDim.x >= ntile)
+            flush(bwd_layer_part(gridDim.x, blockIdx.x, done));
         asm volatile("tcgen05.fence::before_thread_sync;");
     }
-
-    // bias partial: the 32 threads of a channel octet, in a fixed order
-    __syncthreads();
-    {
-        const int part = tid >> 3;
-#pragma unroll
-        for (int t = 0; t < 8; t++) s_bias[part * TC_N + c8 + t] = bsum[t];
-    }
-    __syncthreads();
-    float *out = b.partial + (size_t)blockIdx.x * ((size_t)K * TC_N + TC_N);
-    if (tid < TC_N) {
-        float x = 0.0f;
-        for (int k = 0; k < 32; k++) x += s_bias[k * TC_N + tid];
-        out[(size_t)K * TC_N + tid] = x;
-    }
-    // G rows i: features 0..127 from the first accumulator, 128..191 from the second's lanes 64..127
-    asm volatile("tcgen05.fence::after_thread_sync;");
-    const uint32_t tmem = tmem_base;
-    const int quarter = warp & 3, half = warp >> 2;
-#pragma unroll
-    for (int mt = 0; mt < (KIND == 0 ? 2 : 1); mt++) {
-        const int i = mt * 64 + quarter * 32 + lane;
-#pragma unroll
-        for (int q = 2 * half; q < 2 * half + 2; q++) {
-            float v[16];
-            if (s_ok) {
-                tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + 128 + 64 * mt + q * 16, v);
-            } else {
-#pragma unroll
-                for (int t = 0; t < 16; t++) v[t] = 0.0f;
-            }
-            if (mt == 0 || quarter >= 2) {
-                float4 *dst = reinterpret_cast<float4 *>(out + (size_t)i * TC_N + q * 16);
-#pragma unroll
-                for (int t = 0; t < 16; t += 4) dst[t / 4] = make_float4(v[t], v[t + 1], v[t + 2], v[t + 3]);
-            }
+    if (!s_ok) {
+        // a wait gave up: the rest of the CTA's partial sums are zeros
+        for (; blockIdx.x + done * gridDim.x < ntile; done += kGradTiles - done % kGradTiles) {
+            __syncthreads();
+            flush(bwd_layer_part(gridDim.x, blockIdx.x, done));
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     if (warp == 0) {
         asm volatile("tcgen05.fence::after_thread_sync;");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(256));
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(256));
     }
 }
 
@@ -730,8 +742,6 @@ __host__ __device__ constexpr size_t bwd_layer_smem(int kind)
 }  // namespace
 
 bool linear_tc_supported(int K, int P) { return P == TC_N && (K == 128 || K == 192); }
-
-int bwd_layer_ctas(int N) { return std::max(1, std::min((N + TC_M - 1) / TC_M, 2 * 152)); }
 
 cudaError_t launch_bwd_layer_tc(const BwdLayerArgs &b, unsigned *status, cudaStream_t st)
 {
