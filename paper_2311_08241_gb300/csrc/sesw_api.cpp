@@ -1420,6 +1420,7 @@ int sesw_get_info(sesw_ctx *c, sesw_info *info)
 {
     if (!c || !info) return SESW_EINVAL;
     if (!c->have_mesh) return fail(c, SESW_ESTATE, "no mesh uploaded");
+    DeviceGuard dg(c->device);       // graph_threads asks the device
     memset(info, 0, sizeof *info);
     info->nv = c->dm.nv;
     info->ne = c->dm.ne;
