@@ -215,6 +215,10 @@ typedef struct sesw_info {
     int32_t launches;        /* kernel launches of one step: persistent SE, one per group of packs that
                                 run the same kernel (a launch runs its packs one after another);
                                 persistent SESM, one per pack; graph mode, M + 1 (SE) */
+    int32_t cluster_blocks;  /* persistent SE: blocks of the thread-block cluster that runs a small mesh (see
+                                SESW_FORM_AUTO), one slot per thread; block_threads, blocks_per_sm,
+                                slots_per_thread and cached are then the cluster's. 0: not a cluster */
+    int32_t reserved;        /* 0 */
 } sesw_info;
 
 /* Create a context on CUDA device `device`, issuing work on `cuda_stream` (a
@@ -254,12 +258,19 @@ int sesw_set_mode(sesw_ctx *ctx, int32_t mode);
 /* Persistent mode: which kernel form each pack (one cooperative launch) runs.
  *   SESW_FORM_AUTO             the register form where a thread holds at most 6 slots, or 7 or
  *                              8 with the vertices' data and compensation terms in shared
- *                              memory; else the streaming form (default)
- *   SESW_FORM_REGISTERS        transports and sums in registers, static slot data in shared
- *                              memory when it fits, else the vertices' data and the low parts of
- *                              the compensated sums (sesw_info.streamed = 0)
+ *                              memory; else the streaming form (default). The SE scheme of a single
+ *                              mesh of up to 16 x 1024 slots (about 5,900 vertices) under the
+ *                              automatic residency (sesw_set_blocks_per_sm) runs in one thread-block
+ *                              cluster instead, which exchanges the elevation through the cluster's
+ *                              distributed shared memory (sesw_info.cluster_blocks)
+ *   SESW_FORM_REGISTERS        transports in registers; the static slot data in tensor memory and
+ *                              the vertices' data in shared memory when they fit (from 6 slots per
+ *                              thread the low parts of the compensated sums too), else read from L2
+ *                              (sesw_info.cached; streamed = 0). SESM: all of it on chip
  *   SESW_FORM_STREAM           transports, sums and static data read from L2 slot by slot,
- *                              corner indices in shared memory when they fit (streamed = 1, else 2)
+ *                              corner indices in shared memory when they fit (streamed = 1, else 2).
+ *                              SESM streams only the static data where a thread then holds at most 7
+ *                              slots (streamed = 1)
  *   SESW_FORM_STREAM_UNCACHED  the streaming form with the corner indices read from L2 too
  *                              (streamed = 2)
  * All forms give bitwise the same results (the per-vertex sums run in a fixed order). A mesh

@@ -789,7 +789,8 @@ static int upload_batch(sesw_ctx *c, const sesw_mesh *meshes, int n)
         }
         TRY(upload(c, &d.pack_patch, pp, "pack_patch"));
         TRY(upload(c, &d.pack_off_d, d.pack_off, "pack_off"));
-        if (n == 1 && packs.size() == 1 && !packs[0].plan.stream && c->blocks_per_sm == 0) {
+        // a residency or a form that the caller names is the kernel with the exchange through L2
+        if (n == 1 && packs.size() == 1 && !packs[0].plan.stream && c->blocks_per_sm == 0 && c->form == SESW_FORM_AUTO) {
             std::vector<int> grp, halo;
             std::vector<unsigned> readers;
             d.cluster = sesw::cluster_plan(hm, packs[0].mx.deg, grp, readers, halo);
@@ -1429,7 +1430,13 @@ int sesw_get_info(sesw_ctx *c, sesw_info *info)
     info->max_patch_slots = c->max_patch_slots;
     info->patch_vertices = c->patch_vertices_used;
     // the persistent plan of the scheme in use (SE until SESM parameters are set)
-    const sesw::PersistentPlan &pl = c->have_params && c->params.scheme == 1 ? c->plan_sesm : c->plan;
+    sesw::PersistentPlan pl = c->have_params && c->params.scheme == 1 ? c->plan_sesm : c->plan;
+    if (!(c->have_params && c->params.scheme == 1) && sesw::takes_cluster(c->dm, c->args)) {
+        pl = sesw::PersistentPlan();
+        pl.threads = c->dm.cluster.threads;
+        pl.slots_per_thread = pl.cached = pl.blocks_per_sm = 1;
+        info->cluster_blocks = c->dm.cluster.blocks;
+    }
     info->block_threads = c->mode == SESW_MODE_PERSISTENT ? pl.threads : graph_threads(c);
     info->mode = c->mode;
     info->blocks_per_sm = c->mode == SESW_MODE_PERSISTENT ? pl.blocks_per_sm : 0;

@@ -411,8 +411,7 @@ cudaError_t launch_persistent(const DevMesh &m, const DevState &s, const StepArg
                               cudaStream_t stream)
 {
     const int extra = s.W != nullptr || s.eta_sum != nullptr;
-    // a small mesh: one cluster (the failure test's silent patch needs the exchange through L2)
-    if (m.cluster.blocks > 0 && a.silent_patch < 0) return launch_cluster(m, s, a, M, parity, nsteps, stream);
+    if (takes_cluster(m, a)) return launch_cluster(m, s, a, M, parity, nsteps, stream);   // a small mesh
     for (const PackGroup &g : groups) {
         cudaError_t e;
         if (g.plan.stream) {
