@@ -124,9 +124,10 @@ typedef struct sesw_mesh {
  *   flags        bit 0 (SESW_FLAG_NO_STABILITY_CHECK): accept parameters whose Courant
  *                bound exceeds the stability limit (the bound is conservative);
  *                bit 1 (SESW_FLAG_TEST_FORCE_TIMEOUT, for testing failure detection):
- *                in SESW_MODE_PERSISTENT patch 0 never publishes its halo values and each
- *                bounded wait gives up after ~1e7 cycles instead of ~1 s, so the step
- *                ends early and sesw_status reports SESW_ETIMEOUT
+ *                in SESW_MODE_PERSISTENT patch 0 publishes no halo values in the last step of
+ *                each launch (the only one of sesw_advance(ctx, 1)) and each bounded wait
+ *                gives up after ~2e7 cycles instead of ~1 s, so the launch ends early and
+ *                sesw_status reports SESW_ETIMEOUT
  *   eta_bound    |eta| above this (m) or a non-finite value sets SESW_EUNSTABLE; <= 0 means 1e4
  *   sesm_beta, sesm_delta, sesm_gamma, sesm_zeta
  *                SESM coefficients of Eq. (4.7); all zero selects beta = 0.281105 and, with

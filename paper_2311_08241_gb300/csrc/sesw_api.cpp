@@ -247,11 +247,10 @@ int enqueue_step(sesw_ctx *c)
 // Baroclinic steps that one launch of the persistent SE kernel takes of the next n: it loads the
 // patches once for all of them (about 20 us per step on the 200k-vertex channel). Bounded to
 // about 512 substeps, where that cost is below a hundredth, so that a launch stays in the
-// milliseconds. Groups that stream their state from L2 take one step per launch, and so does the
-// failure test's silent patch.
+// milliseconds. Groups that stream their state from L2 take one step per launch.
 int steps_per_launch(const sesw_ctx *c, int n)
 {
-    if (c->mode != SESW_MODE_PERSISTENT || c->args.silent_patch >= 0) return 1;
+    if (c->mode != SESW_MODE_PERSISTENT) return 1;
     if (c->params.scheme == 1) {
         for (const auto &pk : c->packs)
             if (pk.plan_sesm.stream && !pk.plan_sesm.teams) return 1;
@@ -1431,7 +1430,7 @@ int sesw_get_info(sesw_ctx *c, sesw_info *info)
     info->patch_vertices = c->patch_vertices_used;
     // the persistent plan of the scheme in use (SE until SESM parameters are set)
     sesw::PersistentPlan pl = c->have_params && c->params.scheme == 1 ? c->plan_sesm : c->plan;
-    if (!(c->have_params && c->params.scheme == 1) && sesw::takes_cluster(c->dm, c->args)) {
+    if (!(c->have_params && c->params.scheme == 1) && c->dm.cluster.blocks > 0) {
         pl = sesw::PersistentPlan();
         pl.threads = c->dm.cluster.threads;
         pl.slots_per_thread = pl.cached = pl.blocks_per_sm = 1;

@@ -97,6 +97,7 @@ __global__ void __launch_bounds__(1024, 1) k_cluster(const CArgs A)
     const int v0 = P.patch_v[p0], nown = P.patch_v[p1] - v0;
     const StepArgs a = P.a;
     const float dt = P.patch_dt[p0];             // one mesh, one substep length
+    const bool silent = a.silent_patch >= p0 && a.silent_patch < p1;   // failure test: sends nothing in the last step
     const uint32_t base = (uint32_t)__cvta_generic_to_shared(smem);
     const uint32_t eta = base + (uint32_t)A.off_eta, rows = base + (uint32_t)P.off_flux;
     const uint32_t dummy = base + (uint32_t)P.off_dummy + 4u * (tid & 31);
@@ -108,7 +109,7 @@ __global__ void __launch_bounds__(1024, 1) k_cluster(const CArgs A)
         reinterpret_cast<float4 *>(smem + P.off_flux)[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     for (int i = tid; i < nown; i += T) {
         s_inv[i] = P.inv_av[v0 + i];
-        s_mask[i] = A.readers[v0 + i];
+        s_mask[i] = silent && P.nsteps == 1 ? 0u : A.readers[v0 + i];
     }
     // threads without a slot hold an all-zero one (see k_persistent)
     SlotData q;
@@ -193,6 +194,8 @@ __global__ void __launch_bounds__(1024, 1) k_cluster(const CArgs A)
             // a step ends: the sums of the next one start from zero
             ms = 0;
             shi = slo = make_float2(0.0f, 0.0f);
+            if (silent && m + 1 + P.M == total)
+                for (int i = tid; i < nown; i += T) s_mask[i] = 0u;
         }
     }
     const uint32_t last = eta + ((total & 1) ? 4u : 0u);

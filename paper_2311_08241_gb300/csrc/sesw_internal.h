@@ -222,7 +222,8 @@ struct StepArgs {
     float ab0, ab1, ab2;            // SESM: AB3 weights (Eq. 4.7)
     float am0, am1, am2, am3;       // SESM: AM4 weights (Eq. 4.7)
     int nonlinear_h;
-    int silent_patch = -1;     // persistent kernel: this patch never publishes its halo values (-1: none; test hook)
+    int silent_patch;          // persistent kernels: this patch publishes no halo values in the last step of a
+                               // launch, the only one of most (-1: none; test hook)
     long long wait_cycles;     // persistent kernel: budget of one bounded wait, in SM clock cycles
     double g64;
 };
@@ -328,8 +329,6 @@ cudaError_t launch_persistent_sesm(const DevMesh &m, const DevState &s, const St
 // without owning them. deg: most incidences of a vertex.
 ClusterPlan cluster_plan(const HostMesh &hm, int deg, std::vector<int> &grp, std::vector<unsigned> &readers,
                          std::vector<int> &halo);
-// Whether an SE launch takes the cluster (the failure test's silent patch needs the exchange through L2).
-inline bool takes_cluster(const DevMesh &m, const StepArgs &a) { return m.cluster.blocks > 0 && a.silent_patch < 0; }
 cudaError_t launch_cluster(const DevMesh &m, const DevState &s, const StepArgs &a, int M, int parity, int nsteps,
                            cudaStream_t stream);
 

@@ -190,7 +190,7 @@ __device__ __forceinline__ void persistent_patch(const PArgs &P, const int p, co
         const bool more = m + 1 < total;
         unsigned long long *xout = P.xb[(m + 1) & 1];
         const unsigned long long tag_out = (unsigned long long)(base + (unsigned)(m + 1)) << 32;
-        const bool publish = more && p != a.silent_patch;
+        const bool publish = more && !(p == a.silent_patch && m + P.M >= total);
         bool bad = false;
         for (int i = tid; i < nown; i += T) {
             float sum = 0.0f, inv;
@@ -411,7 +411,7 @@ cudaError_t launch_persistent(const DevMesh &m, const DevState &s, const StepArg
                               cudaStream_t stream)
 {
     const int extra = s.W != nullptr || s.eta_sum != nullptr;
-    if (takes_cluster(m, a)) return launch_cluster(m, s, a, M, parity, nsteps, stream);   // a small mesh
+    if (m.cluster.blocks > 0) return launch_cluster(m, s, a, M, parity, nsteps, stream);   // a small mesh
     for (const PackGroup &g : groups) {
         cudaError_t e;
         if (g.plan.stream) {

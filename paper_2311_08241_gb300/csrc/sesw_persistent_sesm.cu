@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(kSesmThreads, 2) k_persistent_sesm(PArgs P)
         // vertex pass: eta^{m+1}, then eta_AM^{m+1} for the own slots and the neighbours
         unsigned long long *xout = P.xb[x & 1];
         const unsigned long long tag_out = (unsigned long long)(base + (unsigned)x) << 32;
-        const bool publish = p != a.silent_patch;
+        const bool publish = !(p == a.silent_patch && x + P.M > total);
         bool bad = false;
 #pragma unroll
         for (int k = 0; k < kSesmVpt; k++) {
@@ -400,7 +400,7 @@ __device__ __forceinline__ void sesm_patch(const PArgs &P, const int p, const in
         x++;
         unsigned long long *xout = P.xb[x & 1];
         const unsigned long long tag_out = (unsigned long long)(base + (unsigned)x) << 32;
-        const bool publish = p != a.silent_patch;
+        const bool publish = !(p == a.silent_patch && x + P.M > total);
         const int nv = P.row_vertices, nxt = cur == 2 ? 0 : cur + 1, prv = cur == 0 ? 2 : cur - 1;
         bool bad = false;
         for (int i = tid; i < nown; i += T) {

@@ -82,3 +82,38 @@ def test_other_schemes_and_batches_do_not_report_it(S):
         s.sesw_mesh_upload_batch([mesh, mesh])
         s.sesw_set_params_batch([I.Params(tau=50.0, M=5)] * 2)
         assert s.sesw_get_info()["cluster_blocks"] == 0
+
+
+@pytest.mark.parametrize("steps", [1, 3])
+@pytest.mark.parametrize("scheme,bps,form", [(0, 0, AUTO), (0, 2, AUTO), (0, 3, REGISTERS), (1, 0, AUTO), (1, 2, STREAM)])
+def test_waits_give_up_and_the_context_goes_on(S, scheme, bps, form, steps):
+    """Failure detection in the cluster, in the kernels with the exchange through L2 and in the last of several
+    steps of one launch: one patch (one block of the cluster) publishes nothing in a launch's last step, the
+    waits run out after about 10 ms each, and the same context and kernel then run normal steps, bitwise
+    graph mode's."""
+    import time
+
+    mesh = _mesh(60, 61)
+    p = I.Params(tau=40.0, M=5, scheme=scheme)
+    rng = np.random.default_rng(3)
+    eta, U = 0.3 * rng.standard_normal(mesh.nv), 5.0 * rng.standard_normal((mesh.ne, 2))
+    ref, _ = _run(S, mesh, p, steps=[steps], mode=GRAPH)
+    with S.Subcycle() as s:
+        s.sesw_set_mode(PERSISTENT)
+        s.sesw_set_blocks_per_sm(bps)
+        s.sesw_set_persistent_form(form)
+        s.sesw_mesh_upload(mesh)
+        for _ in range(2):
+            s.sesw_set_params(p, flags=S.SESW_FLAG_TEST_FORCE_TIMEOUT)
+            assert (s.sesw_get_info()["cluster_blocks"] > 0) == (scheme == 0 and bps == 0)
+            s.sesw_set_state(eta, U)
+            t0 = time.perf_counter()
+            s.sesw_advance(steps)
+            assert s.sesw_status() == S.SESW_ETIMEOUT
+            assert time.perf_counter() - t0 < 10.0
+            s.sesw_set_params(p)
+            s.sesw_set_state(eta, U)
+            s.sesw_advance(steps)
+            got = s.sesw_get_state()
+            assert s.sesw_status() == S.SESW_OK
+            _same(ref, got, "after a timeout")
