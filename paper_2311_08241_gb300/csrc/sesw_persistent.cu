@@ -164,6 +164,8 @@ __device__ __forceinline__ void persistent_patch(const PArgs &P, const int p, co
     // one round of interior slots: whole warps of them.)
     const int npre = nint >= T ? (nint / T) * T : nint & ~31;
     const int total = P.M * P.nsteps;
+    // substeps below it publish: all but the last, for the failure test's patch none of the last step
+    const int publish_end = p == a.silent_patch ? total - P.M : total - 1;
     for (int m = 0, ms = 0; m < total; m++) {
         if (m == 0) {
             elements(0, nsp);    // every halo elevation is in shared memory
@@ -190,7 +192,7 @@ __device__ __forceinline__ void persistent_patch(const PArgs &P, const int p, co
         const bool more = m + 1 < total;
         unsigned long long *xout = P.xb[(m + 1) & 1];
         const unsigned long long tag_out = (unsigned long long)(base + (unsigned)(m + 1)) << 32;
-        const bool publish = more && !(p == a.silent_patch && m + P.M >= total);
+        const bool publish = m < publish_end;
         bool bad = false;
         for (int i = tid; i < nown; i += T) {
             float sum = 0.0f, inv;

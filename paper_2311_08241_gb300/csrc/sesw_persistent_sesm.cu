@@ -108,6 +108,7 @@ __global__ void __launch_bounds__(kSesmThreads, 2) k_persistent_sesm(PArgs P)
     // (the exchange's tags), m those of the running step, whose closing pass (m = M) is the momentum
     // update of its last substep.
     const int total = P.M * P.nsteps;
+    const int last_publish = p == a.silent_patch ? total - P.M : total;   // failure test: none in the last step
     for (int x = 0, m = 0; x <= total; m++) {
         const bool vertex = m < P.M;
         if (m == 0) {
@@ -165,7 +166,7 @@ __global__ void __launch_bounds__(kSesmThreads, 2) k_persistent_sesm(PArgs P)
         // vertex pass: eta^{m+1}, then eta_AM^{m+1} for the own slots and the neighbours
         unsigned long long *xout = P.xb[x & 1];
         const unsigned long long tag_out = (unsigned long long)(base + (unsigned)x) << 32;
-        const bool publish = !(p == a.silent_patch && x + P.M > total);
+        const bool publish = x <= last_publish;
         bool bad = false;
 #pragma unroll
         for (int k = 0; k < kSesmVpt; k++) {
@@ -366,6 +367,7 @@ __device__ __forceinline__ void sesm_patch(const PArgs &P, const int p, const in
     // x counts the substeps of the launch (the exchange's tags); ms those of the running step, whose
     // closing pass (ms = M) is the momentum update of its last substep
     const int total = P.M * P.nsteps;
+    const int last_publish = p == a.silent_patch ? total - P.M : total;   // failure test: none in the last step
     int cur = 0;                      // level of hist with eta^m
     for (int x = 0, ms = 0; x <= total; ms++) {
         const bool vertex = ms < P.M;
@@ -400,7 +402,7 @@ __device__ __forceinline__ void sesm_patch(const PArgs &P, const int p, const in
         x++;
         unsigned long long *xout = P.xb[x & 1];
         const unsigned long long tag_out = (unsigned long long)(base + (unsigned)x) << 32;
-        const bool publish = !(p == a.silent_patch && x + P.M > total);
+        const bool publish = x <= last_publish;
         const int nv = P.row_vertices, nxt = cur == 2 ? 0 : cur + 1, prv = cur == 0 ? 2 : cur - 1;
         bool bad = false;
         for (int i = tid; i < nown; i += T) {
