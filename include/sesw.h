@@ -191,7 +191,9 @@ typedef struct sesw_info {
                                 chip (vertices' data in shared memory, slots' in tensor memory; the
                                 SESM kernel: all in shared memory), 2 when all but some of the slots'
                                 forcing and corner indices does, the low parts of the compensated sums
-                                in shared memory (large patches); 0: read from L2; streaming kernels (streamed != 0): 1 when the
+                                in shared memory (large patches); 0: read from L2 (also where a vertex has more
+                                than 16 triangles: the places of its fluxes beyond eight are looked up there,
+                                all else is where it would be); streaming kernels (streamed != 0): 1 when the
                                 vertices' data lives in shared memory */
     int32_t nbasin;          /* meshes in the uploaded batch (1 for sesw_mesh_upload) */
     double courant_max;      /* estimated largest substep Courant number sqrt(gH kappa^2) dt

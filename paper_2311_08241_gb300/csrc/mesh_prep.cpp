@@ -604,6 +604,7 @@ int build_halos(HostMesh &hm, std::string &err)
     hm.halo_v.clear();
     hm.slot_l.assign(hm.nslot, make_ushort4(0, 0, 0, 0));
     hm.slot_f.assign(hm.nslot, make_uint2(0xffffffffu, 0x7fffffffu));
+    hm.v_over.assign(hm.patch_v[np], 0u);
     hm.max_patch_local = 0;
     hm.max_patch_halo = 0;
     hm.max_patch_csr = 0;
@@ -641,18 +642,23 @@ int build_halos(HostMesh &hm, std::string &err)
             }
             hm.slot_l[s] = make_ushort4(l[0], l[1], l[2], 0);
         }
-        // where each corner's flux goes: the own vertex it belongs to and its place in that
-        // vertex's incidence order, 21 bits per corner (HostMesh::slot_f)
-        for (int v = vlo; v < vhi; v++)
-            for (int k = hm.vcsr_off[v]; k < hm.vcsr_off[v + 1] && k - hm.vcsr_off[v] < 16; k++) {
+        // where each corner's flux goes: its place in the incidence order of the own vertex it belongs
+        // to, 21 bits per corner (HostMesh::slot_f); fluxes beyond kRowFluxes go to the patch's overflow
+        // quads, a vertex's one after another (HostMesh::v_over)
+        int quads = 0;
+        for (int v = vlo; v < vhi; v++) {
+            const int over = overflow_quads(hm.vcsr_off[v + 1] - hm.vcsr_off[v]);
+            hm.v_over[v] = (uint32_t)(quads & 0xffff) | (uint32_t)over << 16;
+            quads += over;
+            for (int k = hm.vcsr_off[v]; k < hm.vcsr_off[v + 1]; k++) {
                 const uint32_t q = hm.vcsr[k];
                 uint2 &f = hm.slot_f[hm.patch_slot[p] + (int)(q >> 2)];
                 const int c = (int)(q & 3u);
                 uint64_t w = ((uint64_t)f.y << 32) | f.x;
-                const uint64_t e = ((uint64_t)(v - vlo) << 4) | (uint64_t)(k - hm.vcsr_off[v]);
-                w = (w & ~(0x1fffffull << (21 * c))) | (e << (21 * c));
+                w = (w & ~(0x1fffffull << (21 * c))) | ((uint64_t)(k - hm.vcsr_off[v]) << (21 * c));
                 f = make_uint2((uint32_t)w, (uint32_t)(w >> 32));
             }
+        }
         hm.halo_v.insert(hm.halo_v.end(), halo.begin(), halo.end());
         hm.patch_halo[p + 1] = (int)hm.halo_v.size();
         hm.max_patch_local = std::max(hm.max_patch_local, nloc);

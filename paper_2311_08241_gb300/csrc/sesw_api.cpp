@@ -526,8 +526,12 @@ static void make_packs(const sesw::HostMesh &hm, const std::vector<char> &large,
                     pk.mx.halo = std::max(pk.mx.halo, nhq);
                     pk.mx.local = std::max(pk.mx.local, nvq + nhq);
                     pk.mx.csr = std::max(pk.mx.csr, hm.vcsr_off[hm.patch_v[q + 1]] - hm.vcsr_off[hm.patch_v[q]]);
-                    for (int v = hm.patch_v[q]; v < hm.patch_v[q + 1]; v++)
+                    int over = 0;
+                    for (int v = hm.patch_v[q]; v < hm.patch_v[q + 1]; v++) {
                         pk.mx.deg = std::max(pk.mx.deg, hm.vcsr_off[v + 1] - hm.vcsr_off[v]);
+                        over += sesw::overflow_quads(hm.vcsr_off[v + 1] - hm.vcsr_off[v]);
+                    }
+                    pk.mx.over = std::max(pk.mx.over, over);
                 }
             const bool streamed = kform == SESW_FORM_STREAM || kform == SESW_FORM_STREAM_UNCACHED;
             const int idx_mode = kform == SESW_FORM_STREAM_UNCACHED ? 0 : -1;
@@ -607,6 +611,7 @@ static std::vector<sesw::PackGroup> make_groups(const std::vector<sesw::PackPlan
             mx.halo = std::max(mx.halo, pk.mx.halo);
             mx.csr = std::max(mx.csr, pk.mx.csr);
             mx.deg = std::max(mx.deg, pk.mx.deg);
+            mx.over = std::max(mx.over, pk.mx.over);
             const int bps = pk.plan.blocks_per_sm;
             sesw::PersistentPlan np = pk.plan.stream ? sesw::persistent_plan_stream(mx, bps, pk.plan.stream == 2 ? 0 : -1)
                                                      : sesw::persistent_plan(mx, bps);
@@ -812,6 +817,7 @@ static int upload_batch(sesw_ctx *c, const sesw_mesh *meshes, int n)
         TRY(upload(c, &d.halo_v, hm.halo_v, "halo_v"));
         TRY(upload(c, &d.slot_l, hm.slot_l, "slot_l"));
         TRY(upload(c, &d.slot_f, hm.slot_f, "slot_f"));
+        TRY(upload(c, &d.v_over, hm.v_over, "v_over"));
         d.max_patch_local = hm.max_patch_local;
         d.max_patch_vertices = hm.max_patch_vertices;
         d.max_patch_halo = hm.max_patch_halo;
@@ -1440,7 +1446,7 @@ int sesw_get_info(sesw_ctx *c, sesw_info *info)
     info->mode = c->mode;
     info->blocks_per_sm = c->mode == SESW_MODE_PERSISTENT ? pl.blocks_per_sm : 0;
     info->slots_per_thread = c->mode == SESW_MODE_PERSISTENT ? pl.slots_per_thread : 0;
-    info->cached = c->mode == SESW_MODE_PERSISTENT ? pl.cached : 0;
+    info->cached = c->mode == SESW_MODE_PERSISTENT && !pl.over16 ? pl.cached : 0;
     info->streamed = c->mode == SESW_MODE_PERSISTENT ? pl.stream : 0;
     info->courant_max = c->courant_max;
     info->courant_limit = c->have_params ? c->courant_limit : 0.0;

@@ -119,11 +119,11 @@ __global__ void __launch_bounds__(1024, 1) k_cluster(const CArgs A)
         const int s = s0 + (in ? tid : 0);
         const int4 v = P.sv[s];
         const uint2 f = in ? P.sf[s] : make_uint2(0xffffffffu, 0x7fffffffu);
-        // the flux of a corner that its slot's patch owns: the vertex's row, its place in bits 0-3
+        // the flux of a corner that its slot's patch owns: its place in the vertex's row (at most 16)
         auto place = [&](uint32_t e, int vc) {
-            return e == 0x1fffffu ? dummy
-                                  : rows + 16u * (((e & 15u) >> 2) * (uint32_t)P.row_vertices + (uint32_t)(vc - v0)) +
-                                        4u * (e & 3u);
+            return e == 0x1fffffu
+                       ? dummy
+                       : rows + 16u * ((e >> 2) * (uint32_t)P.row_vertices + (uint32_t)(vc - v0)) + 4u * (e & 3u);
         };
         q.g = in ? P.sg[s] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         q.c = in ? P.sk[s] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);

@@ -73,8 +73,9 @@ struct HostMesh {
     std::vector<int> patch_halo;   // [npatch+1] ranges into halo_v
     std::vector<int> halo_v;       // halo vertex ids (new order), sorted per patch
     std::vector<ushort4> slot_l;   // local corner indices of each slot (.w unused)
-    std::vector<uint2> slot_f;     // per corner 21 bits (corner 0 lowest): own local vertex << 4 | the corner's
-                                   // place in that vertex's incidences; all ones: not an own vertex (or place > 15)
+    std::vector<uint2> slot_f;     // per corner 21 bits (corner 0 lowest): the corner's place in its vertex's
+                                   // incidences; all ones: not an own vertex
+    std::vector<uint32_t> v_over;  // per vertex: first (16 bits) and number of its overflow quads in its patch
     int max_patch_local = 0;       // max n_own + n_halo
     int max_patch_halo = 0;        // max n_halo
     int max_patch_csr = 0;         // max incidence entries of one patch's own vertices
@@ -152,6 +153,7 @@ struct DevMesh {
     int *halo_v = nullptr;
     ushort4 *slot_l = nullptr;
     uint2 *slot_f = nullptr;
+    uint32_t *v_over = nullptr;
     int max_patch_local = 0, max_patch_vertices = 0, max_patch_halo = 0, max_patch_csr = 0;
     // small meshes: the cluster's plan, the patch ranges of its blocks, the blocks that read each vertex,
     // the number of vertices that each block reads and does not own
@@ -270,13 +272,21 @@ struct PersistentPlan {
     int stream = 0;             // state and static data in global memory (the streaming kernels):
                                 // 1 with the corner indices in shared memory, 2 without
     int blocks_per_sm = 1;
+    int wide_rows = 1;          // the kernels that run teams: flux rows of the largest degree (up to 16)
+    bool over16 = false;        // the register kernel with a vertex of more than 16 triangles
     size_t smem = 0;
 };
 // Largest patch of a pack: what its shared-memory layout and its plan depend on.
 struct PatchMax {
     int slots = 0, local = 0, vertices = 0, halo = 0, csr = 0;
     int deg = 0;   // most incidences (triangle corners) of one vertex
+    int over = 0;  // overflow quads of one patch
 };
+// The persistent kernels keep a row of corner fluxes for each own vertex in shared memory, of the largest
+// degree up to 16 where that fits and of kRowFluxes where it does not; the fluxes of a vertex with more triangles
+// go on in quads of four of the patch's overflow area, so that a few such vertices cost the others no space.
+constexpr int kRowFluxes = 8;
+inline int overflow_quads(int deg) { return deg > kRowFluxes ? (deg - kRowFluxes + 3) / 4 : 0; }
 // One cooperative launch of a step: blocks [base, base + nblocks) of pack_patch, with the
 // plans of both schemes for its largest patch (the SESM plan may be empty).
 struct PackPlan {

@@ -87,8 +87,7 @@ __device__ __forceinline__ void persistent_patch(const PArgs &P, const int p, co
     for (int i = tid; i < nown; i += T) seta[i] = P.eta_in[v0 + i];
     for (int i = tid; i < nhalo; i += T) seta[nown + i] = P.eta_in[P.halo_v[hb + i]];
     if (CACHED) {
-        float4 *rows = reinterpret_cast<float4 *>(smem_raw + P.off_flux);
-        for (int i = tid; i < P.row_quads * P.row_vertices; i += T) rows[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        clear_rows(P, smem_raw, v0, nown, tid, T);
         for (int i = tid; i < nown; i += T) s_inv[i] = P.inv_av[v0 + i];
         for (int i = tid; i < nhalo; i += T) s_halo[i] = P.halo_v[hb + i];
     }
@@ -114,9 +113,9 @@ __device__ __forceinline__ void persistent_patch(const PArgs &P, const int p, co
             q.a1 = team + 4u * l.y;
             q.a2 = team + 4u * l.z;
             const uint2 f = in ? P.sf[s] : make_uint2(0xffffffffu, 0x7fffffffu);
-            q.f0 = flux_place(P, team, dummy, f.x & 0x1fffffu);
-            q.f1 = flux_place(P, team, dummy, (f.x >> 21) | ((f.y & 0x3ffu) << 11));
-            q.f2 = flux_place(P, team, dummy, (f.y >> 10) & 0x1fffffu);
+            q.f0 = flux_place(P, team, dummy, f.x & 0x1fffffu, v0, l.x);
+            q.f1 = flux_place(P, team, dummy, (f.x >> 21) | ((f.y & 0x3ffu) << 11), v0, l.y);
+            q.f2 = flux_place(P, team, dummy, (f.y >> 10) & 0x1fffffu, v0, l.z);
             TS::store(tm, j, q);
             if (TS::kFluxShared && i < nsp) {
                 *reinterpret_cast<uint32_t *>(smem_raw + P.off_f01 + 4 * i) = (q.f0 >> 2) | (q.f1 << 14);
@@ -197,12 +196,7 @@ __device__ __forceinline__ void persistent_patch(const PArgs &P, const int p, co
         for (int i = tid; i < nown; i += T) {
             float sum = 0.0f, inv;
             if (CACHED) {
-                // the vertex's fluxes in incidence order, zeros behind the last
-                uint32_t row = team + (uint32_t)P.off_flux + 16u * (uint32_t)i;
-                for (int k = 0; k < P.row_quads; k++, row += 16u * (uint32_t)P.row_vertices) {
-                    const float4 c = lds4(row);
-                    sum = __fadd_rn(__fadd_rn(__fadd_rn(__fadd_rn(sum, c.x), c.y), c.z), c.w);
-                }
+                sum = row_flux_sum<(SPT >= 7)>(P, team, v0, i);
                 inv = s_inv[i];
             } else {
                 const int k1 = P.vcsr_off[v0 + i + 1];
@@ -365,12 +359,17 @@ PersistentPlan persistent_plan(const PatchMax &m, int blocks_per_sm)
         for (int spt = 1; spt <= 8; spt++) {
             const int t = std::max(32, ((m.slots + spt - 1) / spt + 31) / 32 * 32);
             if (t > max_threads || !persistent_kernel(spt, 0, cached, 0)) continue;
-            if (cached && m.deg > 16) break;   // HostMesh::slot_f
             const unsigned cols = cached ? tmem_columns(teams * t, tmem_words(spt)) : 0u;
-            const size_t team_smem = se_layout(m, spt, cached).total;
-            size_t smem = teams * team_smem;
-            if (cached) smem = std::max(smem, tmem_smem_floor(cols, (size_t)smem_sm));
-            if (smem > budget || cols > 512u) break;
+            // rows of the largest degree where they fit, else rows of kRowFluxes and overflow quads
+            int wide = 1;
+            size_t team_smem = 0, smem = 0;
+            for (; wide >= 0; wide--) {
+                team_smem = se_layout(m, spt, cached, wide).total;
+                smem = teams * team_smem;
+                if (cached) smem = std::max(smem, tmem_smem_floor(cols, (size_t)smem_sm));
+                if (smem <= budget) break;
+            }
+            if (wide < 0 || cols > 512u) break;
             // every variant the plan may launch must be able to run
             bool fits = true;
             for (int nonlin = 0; nonlin < 2 && fits; nonlin++)
@@ -388,6 +387,8 @@ PersistentPlan persistent_plan(const PatchMax &m, int blocks_per_sm)
             plan.slots_per_thread = spt;
             plan.threads = t;
             plan.cached = cached ? (spt <= 5 ? 1 : 2) : 0;
+            plan.wide_rows = wide;
+            plan.over16 = cached && m.deg > 16;
             plan.teams = teams;
             plan.team_smem = (int)team_smem;
             plan.tmem_cols = (int)cols;
@@ -423,7 +424,7 @@ cudaError_t launch_persistent(const DevMesh &m, const DevState &s, const StepArg
             void *fn = persistent_kernel(g.plan.slots_per_thread, a.nonlinear_h, g.plan.cached, extra);
             if (!fn) return cudaErrorInvalidValue;
             PArgs P = make_pargs(m, s, a, M, parity, g.mx);
-            set_layout(P, se_layout(g.mx, g.plan.slots_per_thread, g.plan.cached), g.mx);
+            set_layout(P, se_layout(g.mx, g.plan.slots_per_thread, g.plan.cached, g.plan.wide_rows), g.mx);
             P.pack_first = g.first;
             P.pack_last = g.last;
             P.nsteps = nsteps;

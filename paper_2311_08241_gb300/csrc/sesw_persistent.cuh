@@ -47,6 +47,7 @@ struct PArgs {
     const int4 *sv;
     const ushort4 *sl;
     const uint2 *sf;           // where each corner's flux goes (DevMesh::slot_f)
+    const uint32_t *vover;     // each vertex's overflow quads (DevMesh::v_over)
     const float4 *sg, *sc;
     const float4 *sk;          // step coefficients of each slot (DevMesh::slot_k)
     const float2 *R;
@@ -69,8 +70,9 @@ struct PArgs {
     int nsteps;                  // baroclinic steps of this launch (k_persistent)
     int npb;                     // patches of the pack (launches of one pack)
     unsigned tmem_cols;          // tensor-memory columns of a block (k_persistent, a power of two)
-    int row_quads, row_vertices; // k_persistent: 16-byte quads of a vertex's row of fluxes; vertices per quad array
-    int off_dummy, off_f01, off_f2, off_slo, off_hist;   // k_persistent: see SeLayout
+    int row_quads, row_vertices; // 16-byte quads of a vertex's row of fluxes; vertices per quad array
+    int over;                    // overflow quads (0: the rows hold every vertex's fluxes)
+    int off_dummy, off_f01, off_f2, off_slo, off_hist, off_over, off_omask;   // k_persistent: see SeLayout
     int team_threads, team_smem; // threads and shared-memory bytes of each patch of a block (k_persistent)
     // shared-memory carve-up (CACHED), in bytes from the dynamic shared base
     int off_flux, off_g, off_c, off_r, off_l, off_off, off_csr, off_inv, off_halo;
@@ -217,13 +219,66 @@ __device__ __forceinline__ void team_sync(int bar, int T)
     asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(T) : "memory");
 }
 
-// Shared-memory address of a flux place (21 bits of HostMesh::slot_f); corners that are not own
-// vertices write to the lane's dummy word.
-__device__ __forceinline__ uint32_t flux_place(const PArgs &P, uint32_t team, uint32_t dummy, uint32_t e)
+// Shared-memory address of a corner's flux: place e (21 bits of HostMesh::slot_f) of the patch's vertex l
+// (v0: its first); corners that are not own vertices write to the lane's dummy word.
+__device__ __forceinline__ uint32_t flux_place(const PArgs &P, uint32_t team, uint32_t dummy, uint32_t e, int v0,
+                                               uint32_t l)
 {
-    return e == 0x1fffffu ? dummy
-                          : team + (uint32_t)P.off_flux +
-                                16u * (((e & 15u) >> 2) * (uint32_t)P.row_vertices + (e >> 4)) + 4u * (e & 3u);
+    if (e == 0x1fffffu) return dummy;
+    if (e < 4u * (uint32_t)P.row_quads)
+        return team + (uint32_t)P.off_flux + 16u * ((e >> 2) * (uint32_t)P.row_vertices + l) + 4u * (e & 3u);
+    return team + (uint32_t)P.off_over + 16u * (P.vover[v0 + (int)l] & 0xffffu) + 4u * (e - (uint32_t)kRowFluxes);
+}
+
+// Clear the flux rows and overflow quads, and mark the own vertices that have any: one bit per vertex, so
+// that a vertex pass looks at a vertex's overflow only where there is some. By the T threads of a team, which the
+// caller synchronises afterwards.
+__device__ __forceinline__ void clear_rows(const PArgs &P, unsigned char *smem_raw, int v0, int nown, int tid, int T)
+{
+    const float4 z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    float4 *rows = reinterpret_cast<float4 *>(smem_raw + P.off_flux);
+    for (int i = tid; i < P.row_quads * P.row_vertices; i += T) rows[i] = z;
+    if (P.over == 0) return;
+    float4 *over = reinterpret_cast<float4 *>(smem_raw + P.off_over);
+    unsigned *mask = reinterpret_cast<unsigned *>(smem_raw + P.off_omask);
+    for (int i = tid; i < P.over; i += T) over[i] = z;
+    const unsigned in_row = (unsigned)(P.row_quads - kRowFluxes / 4);      // of the quads that v_over counts
+    for (int i = tid; i < ((nown + 31) & ~31); i += T) {
+        const unsigned m = __ballot_sync(0xffffffffu, i < nown && P.vover[v0 + min(i, nown - 1)] >> 16 > in_row);
+        if ((i & 31) == 0) mask[i >> 5] = m;
+    }
+}
+
+__device__ __forceinline__ float add4(float sum, const float4 c)
+{
+    return __fadd_rn(__fadd_rn(__fadd_rn(__fadd_rn(sum, c.x), c.y), c.z), c.w);
+}
+
+// The sum of own vertex i's fluxes in incidence order (zeros behind the last). The first eight have both loads
+// in flight before the sums (four steps of the 200k-vertex channel: 401 us in the loop, 380 us), but not in kernels
+// without registers to spare (TIGHT: 7 slots per thread, sphere 1375 us in the loop, 1402 us).
+template <bool TIGHT>
+__device__ __forceinline__ float row_flux_sum(const PArgs &P, uint32_t team, int v0, int i)
+{
+    uint32_t row = team + (uint32_t)P.off_flux + 16u * (uint32_t)i;
+    const uint32_t step = 16u * (uint32_t)P.row_vertices;
+    float sum = 0.0f;
+    if (TIGHT) {
+        for (int k = 0; k < P.row_quads; k++, row += step) sum = add4(sum, lds4(row));
+    } else {
+        const float4 a = lds4(row), b = lds4(row + step);
+        sum = add4(add4(sum, a), b);
+        if (P.row_quads > 2) {
+            sum = add4(sum, lds4(row + 2u * step));
+            if (P.row_quads > 3) sum = add4(sum, lds4(row + 3u * step));
+        }
+    }
+    if (P.over && (lds_u32(team + (uint32_t)P.off_omask + 4u * (uint32_t)(i >> 5)) >> (i & 31)) & 1u) {
+        const uint32_t o = __ldg(P.vover + v0 + i);
+        for (uint32_t k = (uint32_t)P.row_quads - kRowFluxes / 4; k < o >> 16; k++)
+            sum = add4(sum, lds4(team + (uint32_t)P.off_over + 16u * ((o & 0xffffu) + k)));
+    }
+    return sum;
 }
 
 // A slot's static data: gradients, step coefficients (DevMesh::slot_k), forcing, and the
@@ -534,6 +589,8 @@ inline PArgs make_pargs(const DevMesh &m, const DevState &s, const StepArgs &a, 
     P.sv = m.slot_v;
     P.sl = m.slot_l;
     P.sf = m.slot_f;
+    P.vover = m.v_over;
+    P.over = 0;
     P.sg = m.slot_g;
     P.sc = m.slot_c;
     P.sk = m.slot_k;
@@ -580,17 +637,23 @@ inline PArgs make_pargs(const DevMesh &m, const DevState &s, const StepArgs &a, 
 
 // Shared memory of one team, from its largest patch: elevation of own and halo vertices; the
 // fluxes, then 32 dummy words; 1/A_v and halo ids; from 5 slots per thread the flux places, from
-// 6 the low parts of the compensated sums. Vertex-major fluxes (cached): each own vertex has a row
-// of one word per incidence (4 words per quad, quad k of all vertices in array k), which the
+// 6 the low parts of the compensated sums; where a vertex has more than kRowFluxes triangles, the
+// overflow quads and the vertices' marks. Vertex-major fluxes (cached): each own vertex has a row
+// of 8 to 16 words (quad k of all vertices in array k), which the
 // element pass fills and the vertex pass reads 16 bytes at a time, in the place of an
 // index row and eight dependent 4-byte reads (the reads' bank conflicts kept the
-// shared-memory pipe busy longer than the element pass). Not cached: three words per slot.
+// shared-memory pipe busy longer than the element pass). Rows as wide as the largest degree gave
+// every vertex that width: a level-8 sphere with a vertex of nine triangles took 264 KB and left the chip
+// (four steps of a 468k-vertex basin, every 144th vertex of nine triangles: 1715 us streamed, 1200 us here).
+// Not cached: three words per slot.
 struct SeLayout {
-    size_t flux, dummy, inv, halo, f01, f2, slo, hist, total;
-    int quads;
+    size_t flux, dummy, inv, halo, f01, f2, slo, hist, over, omask, total;
+    int quads, nover;            // width of the rows; overflow quads beside them
 };
 
-inline SeLayout se_layout(const PatchMax &m, int spt, int cached)
+// wide: rows for the largest degree up to 16, with overflow quads only beyond that; else rows of
+// kRowFluxes.
+inline SeLayout se_layout(const PatchMax &m, int spt, int cached, int wide)
 {
     SeLayout L{};
     const size_t slots = ((size_t)m.slots + 31) & ~(size_t)31;   // whole warps
@@ -600,8 +663,11 @@ inline SeLayout se_layout(const PatchMax &m, int spt, int cached)
         L.total = align16(o + 12 * slots);
         return L;
     }
-    L.quads = std::max(2, (m.deg + 3) / 4);
+    L.quads = wide ? std::min(4, std::max(kRowFluxes / 4, (m.deg + 3) / 4)) : kRowFluxes / 4;
+    L.nover = m.deg > 4 * L.quads ? m.over : 0;
     o += 16 * (size_t)L.quads * (size_t)m.vertices;
+    L.over = o;
+    o += 16 * (size_t)L.nover;
     L.dummy = o;
     o += 128;
     L.inv = o;
@@ -614,15 +680,17 @@ inline SeLayout se_layout(const PatchMax &m, int spt, int cached)
     if (spt >= 5) o = align16(o + 2 * slots);
     L.slo = o;
     if (spt >= 6) o += sizeof(float2) * slots;
+    L.omask = o;
+    if (L.nover > 0) o += 4 * (((size_t)m.vertices + 31) / 32);
     L.total = align16(o);
     return L;
 }
 
 // The SESM teams: elevation (eta_AM) of own and halo vertices, fluxes, vertices' data as above, the
 // three levels of elevation that each own vertex keeps, and U_AB of the slots.
-inline SeLayout sesm_layout(const PatchMax &m)
+inline SeLayout sesm_layout(const PatchMax &m, int wide)
 {
-    SeLayout L = se_layout(m, 1, 1);
+    SeLayout L = se_layout(m, 1, 1, wide);
     L.hist = L.total;
     L.slo = align16(L.hist + 3 * sizeof(float) * (size_t)m.vertices);
     L.total = L.slo + sizeof(float2) * (((size_t)m.slots + 31) & ~(size_t)31);
@@ -639,6 +707,9 @@ inline void set_layout(PArgs &P, const SeLayout &L, const PatchMax &m)
     P.off_f2 = (int)L.f2;
     P.off_slo = (int)L.slo;
     P.off_hist = (int)L.hist;
+    P.off_over = (int)L.over;
+    P.off_omask = (int)L.omask;
+    P.over = L.nover;
     P.row_quads = L.quads;
     P.row_vertices = m.vertices;
 }

@@ -282,10 +282,7 @@ __device__ __forceinline__ void sesm_patch(const PArgs &P, const int p, const in
     float *s_inv = reinterpret_cast<float *>(smem_raw + P.off_inv);
     int *s_halo = reinterpret_cast<int *>(smem_raw + P.off_halo);
     float *hist = reinterpret_cast<float *>(smem_raw + P.off_hist);   // three levels of row_vertices each
-    {
-        float4 *rows = reinterpret_cast<float4 *>(smem_raw + P.off_flux);
-        for (int i = tid; i < P.row_quads * P.row_vertices; i += T) rows[i] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    }
+    clear_rows(P, smem_raw, v0, nown, tid, T);
     for (int i = tid; i < nown; i += T) {
         s_inv[i] = P.inv_av[v0 + i];
         hist[i] = P.eta_in[v0 + i];
@@ -307,9 +304,9 @@ __device__ __forceinline__ void sesm_patch(const PArgs &P, const int p, const in
         q.a0 = team + 4u * l.x;
         q.a1 = team + 4u * l.y;
         q.a2 = team + 4u * l.z;
-        q.f0 = flux_place(P, team, dummy, f.x & 0x1fffffu);
-        q.f1 = flux_place(P, team, dummy, (f.x >> 21) | ((f.y & 0x3ffu) << 11));
-        q.f2 = flux_place(P, team, dummy, (f.y >> 10) & 0x1fffffu);
+        q.f0 = flux_place(P, team, dummy, f.x & 0x1fffffu, v0, l.x);
+        q.f1 = flux_place(P, team, dummy, (f.x >> 21) | ((f.y & 0x3ffu) << 11), v0, l.y);
+        q.f2 = flux_place(P, team, dummy, (f.y >> 10) & 0x1fffffu, v0, l.z);
         SS::store_places(tm, j, q);
         u1[j] = in ? P.U[s] : make_float2(0.0f, 0.0f);
     }
@@ -406,12 +403,7 @@ __device__ __forceinline__ void sesm_patch(const PArgs &P, const int p, const in
         const int nv = P.row_vertices, nxt = cur == 2 ? 0 : cur + 1, prv = cur == 0 ? 2 : cur - 1;
         bool bad = false;
         for (int i = tid; i < nown; i += T) {
-            float sum = 0.0f;
-            uint32_t row = team + (uint32_t)P.off_flux + 16u * (uint32_t)i;
-            for (int k = 0; k < P.row_quads; k++, row += 16u * (uint32_t)nv) {
-                const float4 c = lds4(row);
-                sum = __fadd_rn(__fadd_rn(__fadd_rn(__fadd_rn(sum, c.x), c.y), c.z), c.w);
-            }
+            const float sum = row_flux_sum<false>(P, team, v0, i);
             const float h0 = hist[cur * nv + i];
             const float h1 = ms == 0 ? h0 : hist[prv * nv + i], h2 = ms == 0 ? h0 : hist[nxt * nv + i];
             float e = vertex_eta(h0, sum, s_inv[i]);
@@ -556,7 +548,7 @@ PersistentPlan persistent_plan_sesm_teams(const PatchMax &m, int blocks_per_sm)
         cudaGetLastError();
         return plan;
     }
-    if (m.deg > 16) return plan;   // HostMesh::slot_f
+    if (m.deg > 16) return plan;   // such meshes stream (k_persistent_sesm_stream)
     const int teams = std::min(std::max(blocks_per_sm, 1), kMaxTeams);
     const int max_threads = kSesmTeamThreads / teams / 32 * 32;
     if (smem_optin < 2048 || smem_sm < 4096) return plan;
@@ -565,9 +557,14 @@ PersistentPlan persistent_plan_sesm_teams(const PatchMax &m, int blocks_per_sm)
         const int t = std::max(32, ((m.slots + spt - 1) / spt + 31) / 32 * 32);
         if (t > max_threads) continue;
         const unsigned cols = tmem_columns(teams * t, sesm_words(spt));
-        const size_t team_smem = sesm_layout(m).total;
-        const size_t smem = std::max(teams * team_smem, tmem_smem_floor(cols, (size_t)smem_sm));
-        if (smem > budget || cols > 512u) return plan;
+        int wide = 1;
+        size_t team_smem = 0, smem = 0;
+        for (; wide >= 0; wide--) {
+            team_smem = sesm_layout(m, wide).total;
+            smem = std::max(teams * team_smem, tmem_smem_floor(cols, (size_t)smem_sm));
+            if (smem <= budget) break;
+        }
+        if (wide < 0 || cols > 512u) return plan;
         for (int nonlin = 0; nonlin < 2; nonlin++) {
             void *fn = sesm_teams_kernel(spt, nonlin);
             int occ = 0;
@@ -581,6 +578,7 @@ PersistentPlan persistent_plan_sesm_teams(const PatchMax &m, int blocks_per_sm)
         plan.threads = t;
         plan.cached = 1;
         plan.stream = 1;
+        plan.wide_rows = wide;
         plan.blocks_per_sm = blocks_per_sm;
         plan.teams = teams;
         plan.team_smem = (int)team_smem;
@@ -625,7 +623,7 @@ cudaError_t launch_persistent_sesm(const DevMesh &m, const DevState &s, const St
         P.nsteps = nsteps;
         int grid = pk.nblocks, threads = pl.threads;
         if (pl.teams) {
-            set_layout(P, sesm_layout(pk.mx), pk.mx);
+            set_layout(P, sesm_layout(pk.mx, pl.wide_rows), pk.mx);
             P.tmem_cols = (unsigned)pl.tmem_cols;
             P.team_threads = pl.threads;
             P.team_smem = pl.team_smem;
