@@ -117,3 +117,15 @@ def test_waits_give_up_and_the_context_goes_on(S, scheme, bps, form, steps):
             got = s.sesw_get_state()
             assert s.sesw_status() == S.SESW_OK
             _same(ref, got, "after a timeout")
+
+
+@pytest.mark.parametrize("scheme,bps,form", [(0, 0, AUTO), (0, 2, AUTO), (0, 1, REGISTERS), (1, 2, AUTO), (1, 2, STREAM)])
+@pytest.mark.parametrize("M,steps", [(200, 5), (512, 3), (513, 2), (7, 80)])
+def test_steps_beyond_one_launch(S, scheme, bps, form, M, steps):
+    """More substeps than one launch takes (512), in the cluster and in every kernel that takes several steps."""
+    mesh = _mesh(41, 37)
+    p = I.Params(tau=5.0 * M, M=M, scheme=scheme)
+    ref, _ = _run(S, mesh, p, [1] * steps, GRAPH)
+    got, info = _run(S, mesh, p, [steps], bps=bps, form=form)
+    assert (info["cluster_blocks"] > 0) == (bps == 0 and scheme == 0), info
+    _same(ref, got, f"M {M}, {steps} steps")
