@@ -593,8 +593,11 @@ def run_ensemble(args, world, rank, local):
     if persistent:
         kernels = ("k_persistent", "k_persistent_stream")
         fig = profile_figures("k_persistent_ensemble", kernels, layout=best.label())
-        roofline = roofline_issue(f"k_persistent + k_persistent_stream ({info['npack']} packs in "
-                                  f"{launches_per_step} launches per step)",
+        # the first pack's form; the layouts that stream only the large basins name both kernels
+        names = "k_persistent_stream" if info["streamed"] else "k_persistent"
+        if best.large_form in (S.SESW_FORM_STREAM, S.SESW_FORM_STREAM_UNCACHED) and not info["streamed"]:
+            names += " + k_persistent_stream (large basins)"
+        roofline = roofline_issue(f"{names} ({info['npack']} packs in {launches_per_step} launches per step)",
                                   mean_step_s, fig and fig.get("warp_instructions_per_step"),
                                   fig and fig.get("dram_bytes_per_step"), b_alg_step, sms, sm_max_mhz_of(clk),
                                   per="step")

@@ -241,9 +241,10 @@ int sesw_set_patch_vertices(sesw_ctx *ctx, int32_t patch_vertices);
 /* Execution modes of a baroclinic step.
  *   SESW_MODE_GRAPH       M launches of the substep kernel (one block per patch of
  *                         ~patch_vertices vertices) plus an epilogue, as one CUDA graph
- *   SESW_MODE_PERSISTENT  one cooperative launch per step (per pack of a batch): each
- *                         block keeps its patch's elevation and fluxes in shared memory
- *                         and its transports in registers for all M substeps (patches
+ *   SESW_MODE_PERSISTENT  one cooperative launch (per group of packs of a batch) for a step
+ *                         or several (up to about 512 substeps of one sesw_advance): each
+ *                         patch keeps its elevation and fluxes in shared memory
+ *                         and its transports in registers for all of them (patches
  *                         too large for that stream their transports and static data
  *                         from L2 instead, see sesw_info.streamed), exchanging boundary
  *                         elevation with neighbouring blocks as tagged words through L2
@@ -323,8 +324,10 @@ int sesw_mesh_upload(sesw_ctx *ctx, const sesw_mesh *mesh);
  * bitwise those of its own upload in any mode and layout. In SESW_MODE_PERSISTENT each basin
  * gets the larger of its one-grid patch size and a common size whose static data fits shared
  * memory (basins larger than one grid of those are cut by sesw_set_large_basins); the meshes
- * are packed, largest first, into packs that each fill at most one grid of resident blocks,
- * a step runs one cooperative launch per pack, and the launches of a step are one CUDA graph.
+ * are packed, largest first, into packs that each fill at most one grid of resident blocks.
+ * A cooperative launch runs one pack (SESM) or the packs that run the same kernel (SE), for one step
+ * or, when no pack streams its state, for several steps of one sesw_advance; the launches of
+ * a single step are one CUDA graph.
  * Caller order of every state,
  * forcing and output array is the concatenation of the meshes in order. Errors name
  * the first bad basin. */

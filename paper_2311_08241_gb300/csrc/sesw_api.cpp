@@ -244,9 +244,9 @@ int enqueue_step(sesw_ctx *c)
     return SESW_OK;
 }
 
-// Baroclinic steps that one launch of the persistent SE kernel takes of the next n: it loads the
-// patches once for all of them (about 20 us per step on the 200k-vertex channel). Bounded to
-// about 512 substeps, where that cost is below a hundredth, so that a launch stays in the
+// Baroclinic steps that one launch of a persistent kernel takes of the next n: it loads the
+// patches once for all of them (about 20 us on the 200k-vertex channel). Bounded to about 512
+// substeps (1.2 ms there, of which that load is under 2 %), so that a launch stays in the
 // milliseconds. Groups that stream their state from L2 take one step per launch.
 int steps_per_launch(const sesw_ctx *c, int n)
 {

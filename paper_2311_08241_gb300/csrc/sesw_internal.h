@@ -258,7 +258,8 @@ int diagnostics_blocks(const DevMesh &m);
 cudaError_t launch_diagnostics_basins(const DevMesh &m, const DevState &s, const StepArgs &a, int parity,
                                       double *out, cudaStream_t stream);
 
-// Persistent kernel: one launch per baroclinic step (see sesw_kernels.cu).
+// Persistent kernels (sesw_persistent.cu, sesw_persistent_sesm.cu and their streaming forms): how a pack of
+// patches runs.
 struct PersistentPlan {
     int slots_per_thread = 0;   // 0: not possible for this mesh
     int threads = 0;

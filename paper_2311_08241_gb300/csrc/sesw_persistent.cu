@@ -1,6 +1,6 @@
 // The persistent step kernel of libsesw (sm_103a): one cooperative launch runs all M
-// substeps of Eq. (4.10) of a baroclinic step, with the time-mean transport of Eq.
-// (4.12) and the freshwater flux of Eq. (4.5).
+// substeps of Eq. (4.10) of one or several baroclinic steps, with the time-mean transport of
+// Eq. (4.12) and the freshwater flux of Eq. (4.5).
 #include <type_traits>
 
 #include "sesw_persistent.cuh"

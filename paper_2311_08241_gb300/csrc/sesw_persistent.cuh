@@ -18,8 +18,10 @@ namespace sesw {
 
 namespace {
 
-// The persistent kernels run one cooperative launch per baroclinic step, one block per
-// patch, all blocks resident.
+// A launch of the persistent kernels is cooperative, with every patch of a pack resident: one
+// block per patch (k_persistent_sesm and the streaming kernels) or one team of warps of a
+// block (k_persistent, k_persistent_sesm_teams). It takes n baroclinic steps of M substeps, its
+// substeps counted on from step to step (the streaming kernels: n = 1).
 //
 // Exchange protocol. Every exchanged value (the elevation, or for SESM its AM4
 // combination) is one 64-bit word holding a tag (high
@@ -32,7 +34,7 @@ namespace {
 // neighbour's tag-(m + 1) values; a neighbour writes those only after its own substep
 // m, in which it read the tag-m values (the neighbour relation is symmetric: each patch
 // reads halo values from every patch that reads from it). Between launches, the last
-// block to leave advances the base by M + 1 (one word per pack in the flag buffer), so
+// patch of a pack to leave advances its base by n M + 1 (one word per pack in the flag buffer), so
 // every word left by an earlier launch carries a tag that this launch never waits for
 // and the buffers need no clearing. Tags wrap modulo 2^32; a wrapped tag could only
 // match a word that no launch has rewritten since, and every launch rewrites every word
@@ -444,9 +446,11 @@ inline unsigned tmem_columns(int threads, int words)
 // Shared memory a block must take so that its share of the SM's shared memory is its share of
 // the SM's 512 tensor-memory columns, less the 1 KB that the system reserves per block and at
 // most 1/32 (and 1 KB) of rounding. Blocks of different launches (other contexts, other streams)
-// may share an SM; columns come in units of 32 = 1/16 of the SM, so blocks that fit its shared
-// memory together always find their columns free, and no resident block can wait for columns
-// that another launch holds.
+// may share an SM; columns come in units of 32 = 1/16 of the SM, so blocks of the persistent kernels that
+// fit its shared memory together always find their columns free, and none of them can wait for columns
+// that another persistent launch holds. The surrogate's kernels take columns without this floor (two vertex
+// blocks of the backward pass hold all 512 with 190 KB of shared memory), but their blocks wait for no
+// other block and give their columns back at their end, so a wait for those ends too.
 inline size_t tmem_smem_floor(unsigned cols, size_t smem_per_sm)
 {
     const size_t share = smem_per_sm / 512 * cols;

@@ -1,5 +1,5 @@
-// The SESM step kernel of libsesw (sm_103a): one cooperative launch runs a baroclinic
-// step of the AB3-AM4 substep of Eqs. (4.7)-(4.8), with the time-mean transport of Eq.
+// The SESM step kernels of libsesw (sm_103a): one cooperative launch runs one or several baroclinic
+// steps of the AB3-AM4 substep of Eqs. (4.7)-(4.8), with the time-mean transport of Eq.
 // (4.12) and the freshwater flux of Eq. (4.5).
 #include "sesw_persistent.cuh"
 
@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(kSesmThreads, 2) k_persistent_sesm(PArgs P)
 // (sesw_persistent.cu). U^{m-1} of a slot lives in registers, U_AB^{m-1} in shared memory, U^{m-2}, the
 // sum and the packed addresses (9 words) in tensor memory; the static data (40 B per slot and
 // substep) come from L2. Before, all state streamed from L2 as well (k_persistent_sesm_stream, now
-// for patches beyond this): 408k vertices, two steps, 1003 -> 654 us.
+// for patches beyond this): 408k vertices, two steps, 1003 -> 639 us.
 // (On-chip patches stay with k_persistent_sesm: teams with their static data in tensor memory measured
 // the same, 488 against 490 us for four steps of the 200k-vertex channel.)
 constexpr int kSesmTeamThreads = 1024;   // 64 registers per thread
