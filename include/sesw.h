@@ -293,7 +293,7 @@ int sesw_set_persistent_form(sesw_ctx *ctx, int32_t form);
  * takes the batch's own value, and form -1 (default) the form of sesw_set_persistent_form.
  * With two blocks per SM and the streaming form, for example, a 400k-vertex basin runs 304
  * patches of ~1300 vertices streamed from L2 while the small basins of the same batch keep one
- * block per SM and their static data in shared memory. Results do not depend on this choice
+ * block per SM and their static data on chip. Results do not depend on this choice
  * (bitwise). Takes effect at the next mesh upload. */
 int sesw_set_large_basins(sesw_ctx *ctx, int32_t blocks_per_sm, int32_t form);
 
@@ -322,8 +322,8 @@ int sesw_mesh_upload(sesw_ctx *ctx, const sesw_mesh *mesh);
  * prepared exactly as sesw_mesh_upload would prepare it alone (its own space-filling
  * curve order and patches), and the layouts are concatenated; a basin's results are
  * bitwise those of its own upload in any mode and layout. In SESW_MODE_PERSISTENT each basin
- * gets the larger of its one-grid patch size and a common size whose static data fits shared
- * memory (basins larger than one grid of those are cut by sesw_set_large_basins); the meshes
+ * gets the larger of its one-grid patch size and a common size whose static data fits the
+ * chip (basins larger than one grid of those are cut by sesw_set_large_basins); the meshes
  * are packed, largest first, into packs that each fill at most one grid of resident blocks.
  * A cooperative launch runs one pack (SESM) or the packs that run the same kernel (SE), for one step
  * or, when no pack streams its state, for several steps of one sesw_advance; the launches of
